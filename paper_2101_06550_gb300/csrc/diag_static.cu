@@ -64,12 +64,24 @@ __global__ void __launch_bounds__(kRowThreads) diag_row_kernel(const double* __r
   }
 }
 
-// Sums the row partials in row order; a non-finite input makes both results NaN.
-__global__ void diag_row_final_kernel(const double* __restrict__ part, int ny, double cell, double* mass,
-                                      double* energy) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Sums the row partials with one block, in a fixed order (one thread walking the
+// rows in turn is a chain of load latencies); a non-finite input makes both results NaN.
+__global__ void __launch_bounds__(kRowThreads) diag_row_final_kernel(const double* __restrict__ part, int ny,
+                                                                     double cell, double* mass, double* energy) {
+  double v[3] = {0, 0, 0};
+  for (int j = threadIdx.x; j < ny; j += kRowThreads)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] += part[3 * j + k];
+  __shared__ double s[3][kRowThreads / 32];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    v[k] = warp_sum(v[k]);
+    if ((threadIdx.x & 31) == 0) s[k][threadIdx.x >> 5] = v[k];
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   double a = 0, b = 0, d = 0;
-  for (int j = 0; j < ny; ++j) { a += part[3 * j]; b += part[3 * j + 1]; d += part[3 * j + 2]; }
+  for (int w = 0; w < kRowThreads / 32; ++w) { a += s[0][w]; b += s[1][w]; d += s[2][w]; }
   const double nan = __longlong_as_double(0x7ff8000000000000LL);
   *mass = d != 0.0 ? nan : a * cell;
   *energy = d != 0.0 ? nan : b * cell;
@@ -110,6 +122,6 @@ extern "C" int ch_diagnostics_noalloc(const double* c, int nx, int ny, double lx
   const double dx = lx / nx, dy = ly / ny;
   cudaStream_t st = (cudaStream_t)stream;
   diag_row_kernel<<<ny, kRowThreads, 0, st>>>(c, nx, ny, 0.5 * gamma / (dx * dx), 0.5 * gamma / (dy * dy), part);
-  diag_row_final_kernel<<<1, 32, 0, st>>>(part, ny, dx * dy, mass_out, energy_out);
+  diag_row_final_kernel<<<1, kRowThreads, 0, st>>>(part, ny, dx * dy, mass_out, energy_out);
   return launch_check("ch_diagnostics_noalloc");
 }
