@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "chx_internal.cuh"
+#include "per_system.cuh"
 
 using namespace chx;
 
@@ -50,9 +51,8 @@ constexpr int kU = 8;
 // scratch g (n * batch doubles, interleaved), the result overwrites c.
 
 // Pentadiagonal (order 4).  Factor rows [ralpha, beta, eps, gam, del, q0, q1,
-// G0, G1] over the m = n - 2 rows of the bordered block, then (PER) the 2x2
-// tail inverse of each system.
-template <bool PER>
+// G0, G1] over the m = n - 2 rows of the bordered block.  (The Rewrite variants'
+// sweeps, with factors per system, are per_system.cuh's.)
 __global__ void __launch_bounds__(kThreads) cn_penta_kernel(double* c, double* __restrict__ gs, int n, int batch,
                                                             const double* __restrict__ fac, double s00, double s01,
                                                             double s10, double s11) {
@@ -60,8 +60,7 @@ __global__ void __launch_bounds__(kThreads) cn_penta_kernel(double* c, double* _
   if (s >= batch) return;
   const int m = n - 2;
   const size_t B = (size_t)batch;
-  const size_t fst = PER ? B : 1, fofs = PER ? (size_t)s : 0;
-#define FAC(k, r) __ldg(&fac[((size_t)(k) * m + (r)) * fst + fofs])
+#define FAC(k, r) __ldg(&fac[(size_t)(k) * m + (r)])
   double* pc = c + s;
   double* pg = gs + s;
   double g1 = 0, g2 = 0, t0 = 0, t1 = 0;
@@ -90,13 +89,6 @@ __global__ void __launch_bounds__(kThreads) cn_penta_kernel(double* c, double* _
     }
 #pragma unroll
     for (int u = 0; u < kU; ++u) buf[u] = nxt[u];
-  }
-  if (PER) {
-    const size_t base = (size_t)9 * m * B + (size_t)s;
-    s00 = __ldg(&fac[base]);
-    s01 = __ldg(&fac[base + B]);
-    s10 = __ldg(&fac[base + 2 * B]);
-    s11 = __ldg(&fac[base + 3 * B]);
   }
   const double fm = pc[(size_t)m * B], fl = pc[(size_t)(m + 1) * B];
   const double r0v = fm - t0, r1v = fl - t1;
@@ -143,14 +135,12 @@ __global__ void __launch_bounds__(kThreads) cn_penta_kernel(double* c, double* _
 
 // Tridiagonal (order 2), Thomas with the Sherman-Morrison correction folded
 // into the sweeps as in tri.cu.  Factor rows [rden, a, chat, z, omega].
-template <bool PER>
 __global__ void __launch_bounds__(kThreads) cn_tri_kernel(double* c, double* __restrict__ gs, int n, int batch,
                                                           const double* __restrict__ fac) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= batch) return;
   const size_t B = (size_t)batch;
-  const size_t fst = PER ? B : 1, fofs = PER ? (size_t)s : 0;
-#define FAC(k, r) __ldg(&fac[((size_t)(k) * n + (r)) * fst + fofs])
+#define FAC(k, r) __ldg(&fac[(size_t)(k) * n + (r)])
   double* pc = c + s;
   double* pg = gs + s;
   double d1 = 0, phi = 0;
@@ -369,15 +359,16 @@ extern "C" int cn1d_step(chx_cn1d_plan* p, double* c, int nsteps, void* stream) 
       if (rc) return rc;
       // the refactor records the inner plan's stream; the sweep follows on `st`
       if (p->order == 4)
-        cn_penta_kernel<true><<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, penta_plan_factors(p->penta), 0, 0, 0,
-                                                    0);
+        penta_per_kernel<double, true><<<ceil_div(p->batch, kPerThreads), kPerThreads, 0, st>>>(
+            c, p->d_g, p->n, p->batch, penta_plan_factors(p->penta));
       else
-        cn_tri_kernel<true><<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, tri_plan_factors(p->tri));
+        tri_per_kernel<double, true><<<ceil_div(p->batch, kPerThreads), kPerThreads, 0, st>>>(
+            c, p->d_g, p->n, p->batch, tri_plan_factors(p->tri));
     } else if (p->order == 4) {
-      cn_penta_kernel<false><<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_fac, p->sinv[0], p->sinv[1],
+      cn_penta_kernel<<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_fac, p->sinv[0], p->sinv[1],
                                                    p->sinv[2], p->sinv[3]);
     } else {
-      cn_tri_kernel<false><<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_fac);
+      cn_tri_kernel<<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_fac);
     }
   }
   p->hdr.last_stream = st;

@@ -10,7 +10,10 @@
 //   tail      x_tail = S^{-1} (f_tail - t)   (Eq. first_two)
 //   backward  x_r = g_r - G_r . x_tail - gam_r x_{r+1} - del_r x_{r+2}
 //             (Eq. solve: xhat = E^{-1}(fhat - k x_tail), G = L^{-1} k).
-// Factor arrays per row: [ralpha, beta, eps, gam, del, q0, q1, G0, G1].
+// Factor arrays per row: [ralpha, beta, eps, gam, del, q0, q1, G0, G1].  PER_SYSTEM
+// plans keep y = R^{-T} h in the place of q and take t += y_r g_r, the same
+// number (h^T E^{-1} f = (R^{-T} h) . (L^{-1} f)): y comes out of the forward
+// factorisation pass, q needs a backward one (per_system.cuh).
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -19,6 +22,7 @@
 
 #include "chx_internal.cuh"
 #include "mixed.cuh"
+#include "per_system.cuh"
 
 using namespace chx;
 
@@ -54,7 +58,7 @@ __device__ __forceinline__ int col_of(int r, int o, int n) {
 // Solve kernel.  TIn: storage of f, TW: storage of the sweep intermediate and of
 // x, TC: arithmetic.  For the plain solve all three are the plan dtype and
 // in == work (in place).
-template <typename TIn, typename TW, typename TC, bool PER>
+template <typename TIn, typename TW, typename TC>
 __global__ void __launch_bounds__(kThreads) penta_solve_kernel(const TIn* in, TW* work, int n, int batch,
                                                                const TC* __restrict__ fac, TC s00, TC s01,
                                                                TC s10, TC s11) {
@@ -62,8 +66,7 @@ __global__ void __launch_bounds__(kThreads) penta_solve_kernel(const TIn* in, TW
   if (s >= batch) return;
   const int m = n - 2;
   const size_t B = (size_t)batch;
-  const size_t fst = PER ? B : 1, fofs = PER ? (size_t)s : 0;
-#define FAC(k, r) ldg(&fac[((size_t)(k) * m + (r)) * fst + fofs])
+#define FAC(k, r) ldg(&fac[(size_t)(k) * m + (r)])
   const TIn* pin = in + s;
   TW* pw = work + s;
   TC g1 = 0, g2 = 0, t0 = 0, t1 = 0;
@@ -92,10 +95,6 @@ __global__ void __launch_bounds__(kThreads) penta_solve_kernel(const TIn* in, TW
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) buf[u] = nxt[u];
-  }
-  if (PER) {
-    const size_t base = (size_t)9 * m * B + (size_t)s;
-    s00 = ldg(&fac[base]); s01 = ldg(&fac[base + B]); s10 = ldg(&fac[base + 2 * B]); s11 = ldg(&fac[base + 3 * B]);
   }
   const TC r0v = (TC)pin[(size_t)m * B] - t0, r1v = (TC)pin[(size_t)(m + 1) * B] - t1;
   const TC xt0 = s00 * r0v + s01 * r1v, xt1 = s10 * r0v + s11 * r1v;
@@ -135,47 +134,65 @@ __global__ void __launch_bounds__(kThreads) penta_solve_kernel(const TIn* in, TW
 
 // ---------------------------------------------------------------------------
 // PER_SYSTEM factorisation, one thread per system; coefficients interleaved.
-// Forward pass: LU of E (paper factor steps), G = L^{-1} k and y = R^{-T} h in
-// registers; backward pass: q = L^{-T} y, S = D - q^T k; tail inverse.
+// One forward pass: LU of E (paper factor steps), G = L^{-1} k, y = R^{-T} h and
+// the tail matrix S = D - h^T E^{-1} k = D - y^T G, then the tail inverse.
 // Only rows 0, 1, m-2 and m-1 of E touch the periodic corners (the k columns,
 // the h entries and the wrapped band entries); the rows between take a
 // straight-line path with k = h = 0.
+// Bound by the FP64 pipe: 20 operations and one reciprocal per row, 112 bytes.
+// The next kFU rows' entries are loaded while the current ones are worked on;
+// a batch of 16384 gives every SM only three or four warps, so without that each
+// row waits for memory.  512 x 16384 on a GB300: 1180 -> 643 us, against a
+// version with a second, backward pass for q = L^{-T} y, no loads ahead and the
+// pivot test in FP64.
+constexpr int kFU = 2;
+
 template <typename T>
-__global__ void __launch_bounds__(kThreads) penta_factor_kernel(const double* __restrict__ a,
-                                                                const double* __restrict__ b,
-                                                                const double* __restrict__ c,
-                                                                const double* __restrict__ d,
-                                                                const double* __restrict__ e, int n, int batch,
-                                                                T* fac, int* status) {
+__global__ void __launch_bounds__(kPerThreads) penta_factor_kernel(const double* __restrict__ a,
+                                                                   const double* __restrict__ b,
+                                                                   const double* __restrict__ c,
+                                                                   const double* __restrict__ d,
+                                                                   const double* __restrict__ e, int n, int batch,
+                                                                   T* __restrict__ fac, int* status) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= batch) return;
   const int m = n - 2;
-  const size_t B = (size_t)batch;
+  const size_t B = (size_t)batch, M = (size_t)m * B;
   const double* co[5] = {a + s, b + s, c + s, d + s, e + s};
   T* F = fac + s;
-#define FST(k, r) F[((size_t)(k) * m + (r)) * B]
   const double tol = 1e3 * 2.220446049250313e-16;
   double ga1 = 0, ga2 = 0, de1 = 0, de2 = 0;  // gam/del of rows r-1, r-2
   double G01 = 0, G02 = 0, G11 = 0, G12 = 0;  // G rows r-1, r-2
   double y01 = 0, y02 = 0, y11 = 0, y12 = 0;  // y rows r-1, r-2
+  double S00 = 0, S01 = 0, S10 = 0, S11 = 0;  // accumulates y^T G
   bool bad = false;
-  // one forward row; b0..b4 the row's entries on E-columns r-2..r+2 (0 off E)
-  auto fwd = [&](int r, double b0, double b1, double b2, double b3, double b4, double k0, double k1, double h0,
-                 double h1) {
-    const double ar = b0;
-    const double br = b1 - ar * ga2;
-    const double al = b2 - ar * de2 - br * ga1;
-    const double scale = fabs(b0) + fabs(b1) + fabs(b2) + fabs(b3) + fabs(b4);
-    if (!(fabs(al) > tol * scale)) bad = true;
+  // one forward row; bn the row's entries on E-columns r-2..r+2 (0 off E)
+  auto fwd = [&](int r, const double (&bn)[5], double k0, double k1, double h0, double h1) {
+    const double ar = bn[0];
+    const double br = fma(-ar, ga2, bn[1]);
+    const double al = fma(-br, ga1, fma(-ar, de2, bn[2]));
+    if (!pivot_ok(al, bn)) bad = true;
     const double ra = 1.0 / al;
-    const double ga = (b3 - br * de1) * ra;
-    const double de = b4 * ra;
-    const double G0 = (k0 - ar * G02 - br * G01) * ra;
-    const double G1 = (k1 - ar * G12 - br * G11) * ra;
-    const double y0 = h0 - ga1 * y01 - de2 * y02;
-    const double y1 = h1 - ga1 * y11 - de2 * y12;
-    FST(0, r) = (T)ra; FST(1, r) = (T)br; FST(2, r) = (T)ar; FST(3, r) = (T)ga; FST(4, r) = (T)de;
-    FST(5, r) = (T)y0; FST(6, r) = (T)y1; FST(7, r) = (T)G0; FST(8, r) = (T)G1;
+    const double ga = fma(-br, de1, bn[3]) * ra;
+    const double de = bn[4] * ra;
+    const double G0 = fma(-br, G01, fma(-ar, G02, k0)) * ra;
+    const double G1 = fma(-br, G11, fma(-ar, G12, k1)) * ra;
+    const double y0 = fma(-de2, y02, fma(-ga1, y01, h0));
+    const double y1 = fma(-de2, y12, fma(-ga1, y11, h1));
+    S00 = fma(y0, G0, S00);
+    S01 = fma(y0, G1, S01);
+    S10 = fma(y1, G0, S10);
+    S11 = fma(y1, G1, S11);
+    T* q = F + (size_t)r * B;
+    q[0] = (T)ra;
+    q[M] = (T)br;
+    q[2 * M] = (T)ar;
+    q[3 * M] = (T)ga;
+    q[4 * M] = (T)de;
+    q[5 * M] = (T)y0;
+    q[6 * M] = (T)y1;
+    q[7 * M] = (T)G0;
+    q[8 * M] = (T)G1;
     ga2 = ga1; ga1 = ga; de2 = de1; de1 = de;
     G02 = G01; G01 = G0; G12 = G11; G11 = G1;
     y02 = y01; y01 = y0; y12 = y11; y11 = y1;
@@ -200,44 +217,30 @@ __global__ void __launch_bounds__(kThreads) penta_factor_kernel(const double* __
 #pragma unroll
       for (int o = -2; o <= 2; ++o)
         if (col_of(m + q, o, n) == r) (q ? h1 : h0) += co[o + 2][(size_t)(m + q) * B];
-    fwd(r, bnd[0], bnd[1], bnd[2], bnd[3], bnd[4], k0, k1, h0, h1);
+    fwd(r, bnd, k0, k1, h0, h1);
   };
   const int lo = m < 2 ? m : 2, hi = m - 2 > lo ? m - 2 : lo;  // interior rows [lo, hi)
+  double nxt[kFU][5];  // the next rows' entries
+  auto load = [&](int r0) {
+#pragma unroll
+    for (int u = 0; u < kFU; ++u)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) nxt[u][k] = r0 + u < hi ? co[k][(size_t)(r0 + u) * B] : 0.0;
+  };
+  load(lo);
   for (int r = 0; r < lo; ++r) fwd_corner(r);
-  for (int r = lo; r < hi; ++r) {
-    const size_t o = (size_t)r * B;
-    fwd(r, co[0][o], co[1][o], co[2][o], co[3][o], co[4][o], 0.0, 0.0, 0.0, 0.0);
+  for (int r0 = lo; r0 < hi; r0 += kFU) {
+    double cur[kFU][5];
+#pragma unroll
+    for (int u = 0; u < kFU; ++u)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) cur[u][k] = nxt[u][k];
+    load(r0 + kFU);
+#pragma unroll
+    for (int u = 0; u < kFU; ++u)
+      if (r0 + u < hi) fwd(r0 + u, cur[u], 0.0, 0.0, 0.0, 0.0);
   }
   for (int r = hi; r < m; ++r) fwd_corner(r);
-  double q01 = 0, q02 = 0, q11 = 0, q12 = 0;  // q rows r+1, r+2
-  double be1 = 0, ep2 = 0, ep1 = 0;           // beta_{r+1}, eps_{r+2}, eps_{r+1}
-  double S00 = 0, S01 = 0, S10 = 0, S11 = 0;  // accumulates q^T k
-  auto bwd = [&](int r, bool corner) {
-    const double ra = (double)FST(0, r);
-    const double q0 = ((double)FST(5, r) - be1 * q01 - ep2 * q02) * ra;
-    const double q1 = ((double)FST(6, r) - be1 * q11 - ep2 * q12) * ra;
-    FST(5, r) = (T)q0;
-    FST(6, r) = (T)q1;
-    if (corner) {
-      double k0 = 0, k1 = 0;
-#pragma unroll
-      for (int o = -2; o <= 2; ++o) {
-        const int cc = r + o;
-        if (cc >= 0 && cc < m) continue;
-        const double v = co[o + 2][(size_t)r * B];
-        if (col_of(r, o, n) == m) k0 += v;
-        else k1 += v;
-      }
-      S00 += q0 * k0; S01 += q0 * k1; S10 += q1 * k0; S11 += q1 * k1;
-    }
-    q02 = q01; q01 = q0; q12 = q11; q11 = q1;
-    ep2 = ep1;
-    ep1 = (double)FST(2, r);
-    be1 = (double)FST(1, r);
-  };
-  for (int r = m - 1; r >= hi; --r) bwd(r, true);
-  for (int r = hi - 1; r >= lo; --r) bwd(r, false);
-  for (int r = lo - 1; r >= 0; --r) bwd(r, true);
   double D00 = 0, D01 = 0, D10 = 0, D11 = 0;
 #pragma unroll
   for (int q = 0; q < 2; ++q)
@@ -251,13 +254,12 @@ __global__ void __launch_bounds__(kThreads) penta_factor_kernel(const double* __
   const double A00 = D00 - S00, A01 = D01 - S01, A10 = D10 - S10, A11 = D11 - S11;
   const double det = A00 * A11 - A01 * A10;
   if (!(fabs(det) > tol * (fabs(A00 * A11) + fabs(A01 * A10)))) bad = true;
-  const size_t base = (size_t)9 * m * B;
-  F[base] = (T)(A11 / det);
-  F[base + B] = (T)(-A01 / det);
-  F[base + 2 * B] = (T)(-A10 / det);
-  F[base + 3 * B] = (T)(A00 / det);
+  T* q = F + 9 * M;
+  q[0] = (T)(A11 / det);
+  q[B] = (T)(-A01 / det);
+  q[2 * B] = (T)(-A10 / det);
+  q[3 * B] = (T)(A00 / det);
   if (bad) set_status(status, CHX_ESINGULAR);
-#undef FST
 }
 
 template <typename T>
@@ -291,7 +293,7 @@ void penta_plan_free(chx_penta_plan* p) {
 
 static int launch_per_system_factor(chx_penta_plan* p, const double* a, const double* b, const double* c,
                                     const double* d, const double* e, cudaStream_t st) {
-  const unsigned blk = balanced_block(p->batch), grid = ceil_div(p->batch, blk);
+  const unsigned blk = kPerThreads, grid = ceil_div(p->batch, blk);
   if (p->dtype == CHX_F64)
     penta_factor_kernel<double><<<grid, blk, 0, st>>>(a, b, c, d, e, p->n, p->batch, (double*)p->d_fac,
                                                             p->hdr.d_status);
@@ -391,22 +393,22 @@ extern "C" int penta_cyclic_solve_batched(chx_penta_plan* p, void* rhs, int batc
   const float* S32 = p->sinv32;
   if (refine) {
     launch_penta_refine_ff((double*)rhs, p->d_work32, p->n, batch, p->d_fac32, p->d_coef, S32, st);
+  } else if (p->mode == CHX_COEF_PER_SYSTEM) {
+    const unsigned pgrid = ceil_div(batch, kPerThreads);
+    if (p->dtype == CHX_F64)
+      penta_per_kernel<double, false><<<pgrid, kPerThreads, 0, st>>>((double*)rhs, nullptr, p->n, batch,
+                                                                     (const double*)p->d_fac);
+    else
+      penta_per_kernel<float, false><<<pgrid, kPerThreads, 0, st>>>((float*)rhs, nullptr, p->n, batch,
+                                                                    (const float*)p->d_fac);
   } else if (p->dtype == CHX_F64) {
     double* x = (double*)rhs;
-    if (p->mode == CHX_COEF_PER_SYSTEM)
-      penta_solve_kernel<double, double, double, true><<<grid, blk, 0, st>>>(x, x, p->n, batch,
-                                                                                 (const double*)p->d_fac, 0, 0, 0, 0);
-    else
-      penta_solve_kernel<double, double, double, false><<<grid, blk, 0, st>>>(
-          x, x, p->n, batch, (const double*)p->d_fac, S[0], S[1], S[2], S[3]);
+    penta_solve_kernel<double, double, double><<<grid, blk, 0, st>>>(x, x, p->n, batch, (const double*)p->d_fac, S[0],
+                                                                     S[1], S[2], S[3]);
   } else {
     float* x = (float*)rhs;
-    if (p->mode == CHX_COEF_PER_SYSTEM)
-      penta_solve_kernel<float, float, float, true><<<grid, blk, 0, st>>>(x, x, p->n, batch,
-                                                                              (const float*)p->d_fac, 0, 0, 0, 0);
-    else
-      penta_solve_kernel<float, float, float, false><<<grid, blk, 0, st>>>(
-          x, x, p->n, batch, (const float*)p->d_fac, S32[0], S32[1], S32[2], S32[3]);
+    penta_solve_kernel<float, float, float><<<grid, blk, 0, st>>>(x, x, p->n, batch, (const float*)p->d_fac, S32[0],
+                                                                  S32[1], S32[2], S32[3]);
   }
   p->hdr.last_stream = st;
   return launch_check("penta_cyclic_solve_batched");

@@ -9,7 +9,11 @@
 // correction x = y - phi z is applied inside the single back sweep:
 //   forward   dhat_i = (f_i - a_i dhat_{i-1}) * rden_i,   phi += omega_i dhat_i
 //   backward  y_i = dhat_i - chat_i y_{i+1},              x_i = y_i - phi z_i.
-// Factor arrays per row: [rden, a, chat, z, omega].
+// Factor arrays per row: [rden, a, chat, z, omega].  PER_SYSTEM plans keep zhat =
+// L^{-1} u in the place of z and take x_i = (dhat_i - phi zhat_i) - chat_i x_{i+1},
+// the same numbers, because zhat comes out of the forward factorisation pass
+// and z needs a backward one; omega is then unscaled, with 1 / (1 + v.z) kept
+// as one more value per system (per_system.cuh).
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -17,13 +21,14 @@
 #include <vector>
 
 #include "chx_internal.cuh"
+#include "per_system.cuh"
 
 using namespace chx;
 
 struct chx_tri_plan {
   PlanHdr hdr;
   int n, batch, mode, dtype;
-  void* d_fac;  // SHARED/UNIFORM: 5*n values; PER_SYSTEM: 5*n*batch values (dtype)
+  void* d_fac;  // SHARED/UNIFORM: 5*n values; PER_SYSTEM: (5*n + 1) * batch values (dtype)
 };
 
 namespace {
@@ -31,13 +36,12 @@ namespace {
 constexpr int kThreads = 128;
 constexpr int kUnroll = 8;
 
-template <typename T, bool PER>
+template <typename T>
 __global__ void __launch_bounds__(kThreads) tri_solve_kernel(T* x, int n, int batch, const T* __restrict__ fac) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= batch) return;
   const size_t B = (size_t)batch;
-  const size_t fst = PER ? B : 1, fofs = PER ? (size_t)s : 0;
-#define FAC(k, r) __ldg(&fac[((size_t)(k) * n + (r)) * fst + fofs])
+#define FAC(k, r) __ldg(&fac[(size_t)(k) * n + (r)])
   T* p = x + s;
   T d1 = 0, phi = 0;
   T buf[kUnroll];
@@ -91,59 +95,75 @@ __global__ void __launch_bounds__(kThreads) tri_solve_kernel(T* x, int n, int ba
 #undef FAC
 }
 
-// PER_SYSTEM factorisation: Thomas factors of A', z = A'^{-1} u, weights omega.
+// PER_SYSTEM factorisation in one forward pass: Thomas factors of A', zhat =
+// L^{-1} u (L the lower factor: z = R^{-1} zhat), the weights omega = R^{-T} e_1
+// (less a_1/b_1 on the last row, so that phi = v.y is one dot product) and
+// v.z = omega . zhat.  As for the pentadiagonal factorisation the next rows'
+// entries are loaded ahead.  1024 x 8192 on a GB300: 590 us, and 279 us for the
+// solve; FP64 pipe as in penta.cu, with too few systems to fill it (256 warps).
+constexpr int kFU = 4;
+
 template <typename T>
-__global__ void __launch_bounds__(kThreads) tri_factor_kernel(const double* __restrict__ a,
-                                                              const double* __restrict__ b,
-                                                              const double* __restrict__ c, int n, int batch,
-                                                              T* fac, int* status) {
+__global__ void __launch_bounds__(kPerThreads) tri_factor_kernel(const double* __restrict__ a,
+                                                                 const double* __restrict__ b,
+                                                                 const double* __restrict__ c, int n, int batch,
+                                                                 T* __restrict__ fac, int* status) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= batch) return;
-  const size_t B = (size_t)batch;
-  T* F = fac + s;
-#define FST(k, r) F[((size_t)(k) * n + (r)) * B]
+  const size_t B = (size_t)batch, M = (size_t)n * B;
   const double tol = 1e3 * 2.220446049250313e-16;
   const double a0 = a[s], b0 = b[s], cN = c[(size_t)(n - 1) * B + s];
   bool bad = !(fabs(b0) > 0.0);
   const double rb = bad ? 0.0 : a0 / b0;
-  double ch1 = 0, z1 = 0;
-  for (int i = 0; i < n; ++i) {
-    const double ai = i > 0 ? a[(size_t)i * B + s] : 0.0;
-    const double ci = i < n - 1 ? c[(size_t)i * B + s] : 0.0;
-    double bi = b[(size_t)i * B + s];
-    if (i == 0) bi = 2.0 * b0;
-    if (i == n - 1) bi = bi + a0 * cN / b0;
-    const double den = bi - ai * ch1;
-    if (!(fabs(den) > tol * (fabs(ai) + fabs(bi) + fabs(ci)))) bad = true;
+  double ch1 = 0, z1 = 0, w = 1.0, vz = 0;
+  auto row = [&](int i, double ai, double bi, double ci, double ui, double dw) {
+    const double den = fma(-ai, ch1, bi);
+    if (!pivot_ok(den, {ai, bi, ci})) bad = true;
     const double rd = 1.0 / den;
     const double ch = ci * rd;
-    const double ui = (i == 0 ? -b0 : 0.0) + (i == n - 1 ? cN : 0.0);
-    const double zh = (ui - ai * z1) * rd;
-    FST(0, i) = (T)rd; FST(1, i) = (T)ai; FST(2, i) = (T)ch; FST(3, i) = (T)zh;
+    const double zh = fma(-ai, z1, ui) * rd;
+    const double om = w - dw;
+    vz = fma(om, zh, vz);
+    T* q = fac + s + (size_t)i * B;
+    q[0] = (T)rd;
+    q[M] = (T)ai;
+    q[2 * M] = (T)ch;
+    q[3 * M] = (T)zh;
+    q[4 * M] = (T)om;
+    w = -ch * w;
     ch1 = ch;
     z1 = zh;
+  };
+  double nxt[kFU][3];
+  auto load = [&](int r0) {
+#pragma unroll
+    for (int u = 0; u < kFU; ++u) {
+      const bool in = r0 + u < n - 1;
+      const size_t o = (size_t)(r0 + u) * B + s;
+      nxt[u][0] = in ? a[o] : 0.0;
+      nxt[u][1] = in ? b[o] : 0.0;
+      nxt[u][2] = in ? c[o] : 0.0;
+    }
+  };
+  load(1);
+  row(0, 0.0, 2.0 * b0, c[s], -b0, 0.0);
+  for (int r0 = 1; r0 < n - 1; r0 += kFU) {
+    double cur[kFU][3];
+#pragma unroll
+    for (int u = 0; u < kFU; ++u)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) cur[u][k] = nxt[u][k];
+    load(r0 + kFU);
+#pragma unroll
+    for (int u = 0; u < kFU; ++u)
+      if (r0 + u < n - 1) row(r0 + u, cur[u][0], cur[u][1], cur[u][2], 0.0, 0.0);
   }
-  double zn = 0, zlast = 0, zfirst = 0;
-  for (int i = n - 1; i >= 0; --i) {
-    const double z = (double)FST(3, i) - (double)FST(2, i) * zn;
-    FST(3, i) = (T)z;
-    if (i == n - 1) zlast = z;
-    zfirst = z;
-    zn = z;
-  }
-  const double vz = zfirst - rb * zlast;
+  const size_t last = (size_t)(n - 1) * B + s;
+  row(n - 1, a[last], b[last] + a0 * cN / b0, 0.0, cN, rb);
   const double den = 1.0 + vz;
   if (!(fabs(den) > tol * (1.0 + fabs(vz)))) bad = true;
-  const double rden = 1.0 / den;  // one division, not one per row
-  double w = 1.0;
-  for (int k = 0; k < n; ++k) {
-    double om = w * rden;
-    if (k == n - 1) om -= rb * rden;
-    FST(4, k) = (T)om;
-    w = -(double)FST(2, k) * w;
-  }
+  fac[5 * M + s] = (T)(1.0 / den);
   if (bad) set_status(status, CHX_ESINGULAR);
-#undef FST
 }
 
 }  // namespace
@@ -161,7 +181,7 @@ void tri_plan_free(chx_tri_plan* p) {
 
 static int launch_tri_factor(chx_tri_plan* p, const double* a, const double* b, const double* c,
                              cudaStream_t st) {
-  const unsigned blk = balanced_block(p->batch), grid = ceil_div(p->batch, blk);
+  const unsigned blk = kPerThreads, grid = ceil_div(p->batch, blk);
   if (p->dtype == CHX_F64)
     tri_factor_kernel<double><<<grid, blk, 0, st>>>(a, b, c, p->n, p->batch, (double*)p->d_fac,
                                                           p->hdr.d_status);
@@ -189,7 +209,7 @@ extern "C" int tri_cyclic_factor(chx_tri_plan** plan, int n, int coef_mode, cons
   cudaStream_t st = (cudaStream_t)stream;
   const size_t esz = dtype == CHX_F64 ? sizeof(double) : sizeof(float);
   if (coef_mode == CHX_COEF_PER_SYSTEM) {
-    const size_t cnt = (size_t)5 * n * batch;
+    const size_t cnt = ((size_t)5 * n + 1) * (size_t)batch;
     if (cudaMalloc(&p->d_fac, cnt * esz) != cudaSuccess) {
       cudaGetLastError();
       p->d_fac = nullptr;
@@ -247,16 +267,18 @@ extern "C" int tri_cyclic_solve_batched(chx_tri_plan* p, void* rhs, int batch, v
     return fail(CHX_EINVAL, "tri_cyclic_solve_batched: PER_SYSTEM batch must equal the factor batch %d", p->batch);
   cudaStream_t st = (cudaStream_t)stream;
   const unsigned blk = balanced_block(batch), grid = ceil_div(batch, blk);
-  if (p->dtype == CHX_F64) {
-    if (p->mode == CHX_COEF_PER_SYSTEM)
-      tri_solve_kernel<double, true><<<grid, blk, 0, st>>>((double*)rhs, p->n, batch, (const double*)p->d_fac);
+  if (p->mode == CHX_COEF_PER_SYSTEM) {
+    const unsigned pgrid = ceil_div(batch, kPerThreads);
+    if (p->dtype == CHX_F64)
+      tri_per_kernel<double, false><<<pgrid, kPerThreads, 0, st>>>((double*)rhs, nullptr, p->n, batch,
+                                                                   (const double*)p->d_fac);
     else
-      tri_solve_kernel<double, false><<<grid, blk, 0, st>>>((double*)rhs, p->n, batch, (const double*)p->d_fac);
+      tri_per_kernel<float, false><<<pgrid, kPerThreads, 0, st>>>((float*)rhs, nullptr, p->n, batch,
+                                                                  (const float*)p->d_fac);
+  } else if (p->dtype == CHX_F64) {
+    tri_solve_kernel<double><<<grid, blk, 0, st>>>((double*)rhs, p->n, batch, (const double*)p->d_fac);
   } else {
-    if (p->mode == CHX_COEF_PER_SYSTEM)
-      tri_solve_kernel<float, true><<<grid, blk, 0, st>>>((float*)rhs, p->n, batch, (const float*)p->d_fac);
-    else
-      tri_solve_kernel<float, false><<<grid, blk, 0, st>>>((float*)rhs, p->n, batch, (const float*)p->d_fac);
+    tri_solve_kernel<float><<<grid, blk, 0, st>>>((float*)rhs, p->n, batch, (const float*)p->d_fac);
   }
   p->hdr.last_stream = st;
   return launch_check("tri_cyclic_solve_batched");
