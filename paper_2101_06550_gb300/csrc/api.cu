@@ -30,7 +30,7 @@ int cuda_check(cudaError_t e, const char* what) {
 
 int launch_check(const char* what) { return cuda_check(cudaGetLastError(), what); }
 
-unsigned balanced_block(size_t threads) {
+int sm_count() {
   static int sms[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -39,7 +39,20 @@ unsigned balanced_block(size_t threads) {
     cudaGetLastError();
     n = 152;
   }
-  return threads < (size_t)128 * 16 * n ? 32u : 128u;
+  return n;
+}
+
+unsigned balanced_block(size_t threads) { return threads < (size_t)128 * 16 * sm_count() ? 32u : 128u; }
+
+unsigned one_wave_block(size_t threads) {
+  const int n = sm_count();
+  const size_t nw = (threads + 31) / 32;
+  size_t best = 1, cost = (size_t)-1;
+  for (size_t w = 1; w <= kMaxBlockWarps; ++w) {
+    const size_t c = (((nw + w - 1) / w + n - 1) / n) * w;  // warps on the busiest SM
+    if (c <= cost) cost = c, best = w;
+  }
+  return (unsigned)best * 32;
 }
 
 int hdr_init(PlanHdr* h, uint32_t magic) {

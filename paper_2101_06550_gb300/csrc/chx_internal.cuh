@@ -35,6 +35,14 @@ __device__ __forceinline__ void set_status(int* st, int code) {
   if (st) atomicCAS(st, 0, code);
 }
 
+// The value in an ordinary (per-thread) register.  A DFMA on three of those issues
+// every 16 cycles and SM; one with an immediate or a constant-bank operand every
+// 19, like DADD and DMUL (measured, four warps or more).  The compiler cannot see
+// through the shuffle that the value is the same for the whole warp.
+__device__ __forceinline__ double in_register(double v) {
+  return __shfl_sync(__activemask(), v, threadIdx.x & 31);
+}
+
 inline unsigned ceil_div(size_t a, size_t b) { return (unsigned)((a + b - 1) / b); }
 
 // Threads per block for one-thread-per-system kernels, whose time is set by the
@@ -43,6 +51,17 @@ inline unsigned ceil_div(size_t a, size_t b) { return (unsigned)((a + b - 1) / b
 // 3 on others, 84% balance); single-warp blocks spread the warps to within one
 // of each other (96%).  Many blocks balance by themselves and keep 128.
 unsigned balanced_block(size_t threads);
+int sm_count();  // of the current device
+
+// Threads per block that leave the busiest SM the fewest warps, the largest such
+// block up to kMaxBlockWarps.  The FP64 unit of an SM needs four warps to run at
+// its rate (one warp issues at most one FP64 instruction per 64 cycles, the SM one
+// per 16): the warps of one block start and stay together, single-warp blocks of
+// an SM drift apart until the last ones run alone.  2048 warps (blocks of 14, one
+// per SM): pentadiagonal circulant sweeps 988 us in single-warp blocks, 931 us in
+// these.
+constexpr unsigned kMaxBlockWarps = 16;
+unsigned one_wave_block(size_t threads);
 
 // ---------------------------------------------------------------------------
 // Host FP64 factorisation of one cyclic pentadiagonal system (Secs. 4.2.2-4.2.3).

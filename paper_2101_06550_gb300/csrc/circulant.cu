@@ -1,0 +1,140 @@
+// Host factorisation of symmetric definite circulant band rows (circulant.cuh).
+#include "circulant.cuh"
+
+#include <math.h>
+
+namespace chx {
+namespace {
+
+// A number as the unevaluated sum of two doubles (Dekker, Knuth).  The products
+// pass through a volatile so that the host compiler cannot contract them into the
+// additions that follow.
+struct dd {
+  double hi = 0, lo = 0;
+};
+dd dd_add(dd a, dd b) {
+  const double s = a.hi + b.hi, t = s - a.hi;
+  const double e = ((a.hi - (s - t)) + (b.hi - t)) + (a.lo + b.lo);
+  const double hi = s + e;
+  return dd{hi, e - (hi - s)};
+}
+dd dd_mul(dd a, double b) {
+  volatile double p = a.hi * b;
+  const double hi = p, e = fma(a.hi, b, -hi) + a.lo * b;
+  const double s = hi + e;
+  return dd{s, e - (s - hi)};
+}
+dd dd_mul2(dd a, dd b) {
+  volatile double p = a.hi * b.hi;
+  const double hi = p, e = fma(a.hi, b.hi, -hi) + (a.hi * b.lo + a.lo * b.hi);
+  const double s = hi + e;
+  return dd{s, e - (s - hi)};
+}
+
+}  // namespace
+
+bool circ_pays(int n, int R, int batch, int ops, int closure_ops, double lu_ops) {
+  if (ceil_div(batch, 32) < 4u * (unsigned)sm_count()) return true;
+  return (double)ops * n + (double)closure_ops * R <= lu_ops * n;
+}
+
+bool circ_factor_host(int n, double a_, double b_, double c_, double scale, CircTable* out) {
+  typedef long double ld;
+  if (n < 3 || !isfinite(a_) || !isfinite(b_) || !isfinite(c_) || c_ == 0.0) return false;
+  const ld sign = c_ < 0 ? -1 : 1;
+  const ld a = sign * a_, b = sign * b_, c = sign * c_;
+  // start: the LU factors of the infinite band, whose rows converge to the
+  // spectral factors when the symbol is positive (Bauer's method)
+  double ga1 = 0, ga2 = 0, de1 = 0, de2 = 0, al = 0;
+  {
+    const double as = (double)a, bs = (double)b, cs = (double)c;
+    for (int it = 0; it < 20000; ++it) {
+      const double br = bs - as * ga2;
+      al = cs - as * de2 - br * ga1;
+      if (!(al > 0)) return false;
+      const double ga = (bs - br * de1) / al, de = as / al;
+      const bool done = it > 4 && fabs(ga - ga1) + fabs(de - de1) < 1e-12;
+      ga2 = ga1, ga1 = ga, de2 = de1, de1 = de;
+      if (done) break;
+    }
+  }
+  // Newton (Wilson's method) on q0^2 + q1^2 + q2^2 = c, q0 q1 + q1 q2 = b, q0 q2 = a
+  ld q0 = sqrtl((ld)al), q1 = ga1 * q0, q2 = de1 * q0;
+  ld res = 0;
+  for (int it = 0; it < 60; ++it) {
+    const ld r0 = c - (q0 * q0 + q1 * q1 + q2 * q2), r1 = b - q1 * (q0 + q2), r2 = a - q0 * q2;
+    res = fabsl(r0) + fabsl(r1) + fabsl(r2);
+    if (res <= 4e-19L * c) break;
+    // rows (2 q0, 2 q1, 2 q2), (q1, q0 + q2, q1), (q2, 0, q0) by Cramer's rule
+    const ld s = q0 + q2;
+    const ld det = 2 * q0 * (s * q0) - 2 * q1 * (q1 * q0 - q1 * q2) + 2 * q2 * (-s * q2);
+    if (!(fabsl(det) > 0)) return false;
+    const ld d0 = r0 * (s * q0) - 2 * q1 * (r1 * q0 - q1 * r2) + 2 * q2 * (-s * r2);
+    const ld d1 = 2 * q0 * (r1 * q0 - q1 * r2) - r0 * (q1 * q0 - q1 * q2) + 2 * q2 * (q1 * r2 - r1 * q2);
+    const ld d2 = 2 * q0 * (s * r2) - 2 * q1 * (q1 * r2 - r1 * q2) + r0 * (-s * q2);
+    q0 += d0 / det, q1 += d1 / det, q2 += d2 / det;
+  }
+  if (!(res <= 1e-18L * c) || !(q0 > 0)) return false;
+  const double l1 = (double)(q1 / q0), l2 = (double)(q2 / q0);
+  // both roots inside the unit circle (Schur's conditions), and the sum of L's
+  // coefficients, which the gains of the smoothest modes hang on, known to 2^-39
+  const ld sum = (1.0L + l2) + (ld)l1;
+  if (!(fabs(l2) < 1.0) || !(fabsl((ld)l1) < 1.0L + l2) || !(sum > 0x1p-14L)) return false;
+  const ld lam0 = c + 2 * (a + b);
+  if (!(lam0 > 0)) return false;
+  // 1 / kappa, set so that the mean's gain 1 / lam0 is exact with l1 and l2 as rounded
+  const ld kinv = sum * sum / lam0 * sign;
+  // h from the rounded coefficients, in double-double (a long double is emulated
+  // on some hosts, and this is the loop over rows): h[r + 1] = h_r
+  std::vector<dd> h(n + 3);
+  h[1].hi = 1;
+  for (int r = 1; r <= n + 1; ++r) {
+    h[r + 1] = dd_add(dd_mul(h[r], -l1), dd_mul(h[r - 1], -l2));
+    if (fabs(h[r + 1].hi) < 0x1p-200 && fabs(h[r].hi) < 0x1p-200) break;  // the rest stays 0
+  }
+  int R = n;
+  while (R > 0 && fabs(h[R].hi) < 0x1p-60 && fabs(h[R + 1].hi) < 0x1p-60) --R;
+  R = (R + kCircU) / kCircU * kCircU;
+  if (R > n) R = n;
+  auto H = [&](int j) { return (ld)h[j].hi + (ld)h[j].lo; };
+  // Phi: the closure terms at rows n - 1 and n - 2 for (s1, s2)
+  const ld p00 = 1 - H(n + 1), p01 = (ld)l2 * H(n), p10 = -H(n), p11 = 1 + (ld)l2 * H(n - 1);
+  const ld det = p00 * p11 - p01 * p10;
+  if (!(fabsl(det) > 0)) return false;
+  const ld A[4] = {p11 / det, -p01 / det, -p10 / det, p00 / det};
+  // dot products of the closure terms themselves: sums of h_r h_{r+1}, h_r^2 and h_{r-1} h_r
+  dd q01, q00, qm0;
+  dd prev;
+  for (int r = 0; r < n && r <= R; ++r) {
+    const dd hr = h[r + 1];
+    q01 = dd_add(q01, dd_mul2(hr, h[r + 2]));
+    q00 = dd_add(q00, dd_mul2(hr, hr));
+    qm0 = dd_add(qm0, dd_mul2(h[r], hr));
+    prev = dd_add(prev, dd_mul2(h[r], h[r + 2]));
+  }
+  const ld M[4] = {(ld)q01.hi + q01.lo, -(ld)l2 * ((ld)q00.hi + q00.lo), (ld)prev.hi + prev.lo,
+                   -(ld)l2 * ((ld)qm0.hi + qm0.lo)};
+  out->R = R;
+  out->tab.assign(kCircH + R + 3, 0.0);
+  double* t = out->tab.data();
+  t[0] = -l1, t[1] = -l2, t[2] = (double)(kinv * scale), t[3] = -1.0, t[4] = -2.0;
+  for (int k = 0; k < 4; ++k) t[5 + k] = (double)A[k];
+  t[9] = (double)(A[0] * M[0] + A[1] * M[2]), t[10] = (double)(A[0] * M[1] + A[1] * M[3]);
+  t[11] = (double)(A[2] * M[0] + A[3] * M[2]), t[12] = (double)(A[2] * M[1] + A[3] * M[3]);
+  for (int j = 0; j < R + 3 && j < n + 3; ++j) t[kCircH + j] = h[j].hi + h[j].lo;
+  for (int k = 0; k < (int)out->tab.size(); ++k)
+    if (!isfinite(t[k])) return false;
+  return true;
+}
+
+int circ_upload(const CircTable& t, double** dst, const char* what) {
+  const size_t bytes = t.tab.size() * sizeof(double);
+  if (cudaMalloc(dst, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    *dst = nullptr;
+    return fail(CHX_ENOMEM, "%s: circulant table allocation", what);
+  }
+  return cuda_check(cudaMemcpy(*dst, t.tab.data(), bytes, cudaMemcpyHostToDevice), what);
+}
+
+}  // namespace chx

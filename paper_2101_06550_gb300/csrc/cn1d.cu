@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "chx_internal.cuh"
+#include "circulant.cuh"
 #include "per_system.cuh"
 
 using namespace chx;
@@ -30,6 +31,9 @@ struct chx_cn1d_plan {
   double sigma;
   double* d_fac;  // Constant: penta 9*(n-2), tri 5*n doubles
   double sinv[4];
+  // Constant: the circulant table (scale 2 / kappa), nullptr when sigma is beyond it and the LU factors serve
+  double* d_circ;
+  int circ_rows;
   double* d_g;    // forward-sweep scratch, n * batch doubles
   // Rewrite: per-system matrix entries (order + 1 diagonals of n * batch) and a
   // PER_SYSTEM solver plan holding the per-system factors
@@ -202,6 +206,27 @@ __global__ void __launch_bounds__(kThreads) cn_tri_kernel(double* c, double* __r
 #undef FAC
 }
 
+// Constant mode through the circulant factorisation (circulant.cuh): the scale
+// 2 / kappa rides on the final 2u - c, so a row takes 5 FP64 operations (9 where
+// the closure reaches) for order 4 and 3 (5) for order 2.  1024 x 65536 on a
+// GB300: hyperdiffusion 1207 -> 832 us, diffusion 749 -> 432 us (40 bytes per
+// row are 400 us of HBM there).
+template <int W>
+__global__ void __launch_bounds__(W == 2 ? kMaxBlockWarps * 32 : kThreads) cn_circ_kernel(double* c, double* __restrict__ gs, int n, int batch,
+                                                           const double* __restrict__ tab, int R) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= batch) return;
+  const size_t B = (size_t)batch;
+  double* pc = c + s;
+  double* pg = gs + s;
+  const double sc = in_register(__ldg(tab + 2));
+  circ_sweeps<W>(
+      n, tab, R, [&](int r) { return pc[(size_t)r * B]; }, [](double v) { return v; },
+      [&](int r, double g) { pg[(size_t)r * B] = g; }, [&](int r) { return pg[(size_t)r * B]; },
+      [&](int r) { return pc[(size_t)r * B]; },
+      [&](int r, double y, double cr) { pc[(size_t)r * B] = fma(sc, y, -cr); });
+}
+
 // Rewrite mode: every system's matrix entries, diagonal k of row i at
 // coef[(k * n + i) * batch + s], set to the scheme's implicit coefficients.
 __global__ void cn_reset_matrix_kernel(double* coef, size_t per_diag, int ndiag, double v0, double v1, double v2,
@@ -234,6 +259,7 @@ void* cn1d_inner_plan(chx_cn1d_plan* p) {
 void cn1d_plan_free(chx_cn1d_plan* p) {
   if (!p) return;
   if (p->d_fac) cudaFree(p->d_fac);
+  if (p->d_circ) cudaFree(p->d_circ);
   if (p->d_g) cudaFree(p->d_g);
   if (p->d_coef) cudaFree(p->d_coef);
   if (p->penta) penta_plan_free(p->penta);
@@ -343,6 +369,11 @@ extern "C" int cn1d_plan_create(chx_cn1d_plan** plan, int order, int n, int batc
   }
   rc = cuda_check(cudaMemcpy(p->d_fac, arr, cnt * sizeof(double), cudaMemcpyHostToDevice), "cn1d_plan_create: upload");
   free(arr);
+  CircTable ct;
+  if (!rc && circ_factor_host(n, order == 4 ? v[0] : 0.0, order == 4 ? v[1] : v[0], order == 4 ? v[2] : v[1], 2.0, &ct)) {
+    p->circ_rows = ct.R;
+    rc = circ_upload(ct, &p->d_circ, "cn1d_plan_create");
+  }
   if (rc) { cn1d_plan_free(p); return rc; }
   *plan = p;
   return CHX_OK;
@@ -353,6 +384,7 @@ extern "C" int cn1d_step(chx_cn1d_plan* p, double* c, int nsteps, void* stream) 
   if (!c || nsteps < 0) return fail(CHX_EINVAL, "cn1d_step: null field or nsteps %d < 0", nsteps);
   cudaStream_t st = (cudaStream_t)stream;
   const unsigned blk = balanced_block(p->batch), grid = ceil_div(p->batch, blk);
+  const unsigned cblk = one_wave_block(p->batch), cgrid = ceil_div(p->batch, cblk);
   for (int k = 0; k < nsteps; ++k) {
     if (p->rewrite) {
       int rc = cn1d_reset_and_factor(p, st);
@@ -364,6 +396,11 @@ extern "C" int cn1d_step(chx_cn1d_plan* p, double* c, int nsteps, void* stream) 
       else
         tri_per_kernel<double, true><<<ceil_div(p->batch, kPerThreads), kPerThreads, 0, st>>>(
             c, p->d_g, p->n, p->batch, tri_plan_factors(p->tri));
+    } else if (p->d_circ && circ_pays(p->n, p->circ_rows, p->batch, p->order == 4 ? 5 : 3, p->order, p->order == 4 ? 10.0 : 6.0)) {
+      if (p->order == 4)
+        cn_circ_kernel<2><<<cgrid, cblk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_circ, p->circ_rows);
+      else  // memory-bound: single-warp blocks (432 us; 466 us in one_wave_block's)
+        cn_circ_kernel<1><<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_circ, p->circ_rows);
     } else if (p->order == 4) {
       cn_penta_kernel<<<grid, blk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_fac, p->sinv[0], p->sinv[1],
                                                    p->sinv[2], p->sinv[3]);

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "chx_internal.cuh"
+#include "circulant.cuh"
 #include "mixed.cuh"
 #include "per_system.cuh"
 
@@ -31,6 +32,8 @@ struct chx_penta_plan {
   int n, m, batch, mode, dtype;
   void* d_fac;        // SHARED/UNIFORM: 9*m values; PER_SYSTEM: (9*m + 4) * batch values (dtype)
   double sinv[4];     // SHARED/UNIFORM tail inverse
+  double* d_circ;     // UNIFORM FP64 plans with a symmetric definite row: the circulant table (else nullptr)
+  int circ_rows;
   // FP32 sweeps + double-float residual refinement (SHARED/UNIFORM FP64 plans)
   float* d_fac32;     // 9*m floats
   float2* d_coef;     // 5*n double-float pairs: the rows of A for the residual
@@ -130,6 +133,22 @@ __global__ void __launch_bounds__(kThreads) penta_solve_kernel(const TIn* in, TW
     for (int u = 0; u < kUnroll; ++u) buf[u] = nxt[u];
   }
 #undef FAC
+}
+
+// UNIFORM rows through the circulant factorisation (circulant.cuh), in place.
+// FP64-pipe bound: 5 to 9 operations per row.  1024 x 65536, a = 7e3, on a GB300:
+// 1066 -> 931 us (LU sweeps with bordering, 9 operations, before).
+__global__ void __launch_bounds__(kMaxBlockWarps * 32) penta_circ_kernel(double* x, int n, int batch,
+                                                              const double* __restrict__ tab, int R) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= batch) return;
+  const size_t B = (size_t)batch;
+  double* px = x + s;
+  const double sc = in_register(__ldg(tab + 2));
+  circ_sweeps<2>(
+      n, tab, R, [&](int r) { return px[(size_t)r * B]; }, [](double v) { return v; },
+      [&](int r, double g) { px[(size_t)r * B] = g; }, [&](int r) { return px[(size_t)r * B]; },
+      [](int) { return 0.0; }, [&](int r, double y, double) { px[(size_t)r * B] = y * sc; });
 }
 
 // ---------------------------------------------------------------------------
@@ -283,6 +302,7 @@ const double* penta_plan_factors(const chx_penta_plan* p) { return (const double
 void penta_plan_free(chx_penta_plan* p) {
   if (!p) return;
   if (p->d_fac) cudaFree(p->d_fac);
+  if (p->d_circ) cudaFree(p->d_circ);
   if (p->d_fac32) cudaFree(p->d_fac32);
   if (p->d_coef) cudaFree(p->d_coef);
   if (p->d_work32) cudaFree(p->d_work32);
@@ -363,6 +383,12 @@ extern "C" int penta_cyclic_factor(chx_penta_plan** plan, int n, int coef_mode, 
     }
   }
   free(pf.arr);
+  CircTable ct;
+  if (!rc && dtype == CHX_F64 && coef_mode == CHX_COEF_UNIFORM && a[0] == e[0] && b[0] == d[0] &&
+      circ_factor_host(n, a[0], b[0], c[0], 1.0, &ct)) {
+    p->circ_rows = ct.R;
+    rc = circ_upload(ct, &p->d_circ, "penta_cyclic_factor");
+  }
   if (rc) { penta_plan_free(p); return rc; }
   p->hdr.last_stream = st;
   *plan = p;
@@ -389,6 +415,7 @@ extern "C" int penta_cyclic_solve_batched(chx_penta_plan* p, void* rhs, int batc
     return fail(CHX_EUNSUPPORTED, "penta_cyclic_solve_batched: refine with PER_SYSTEM coefficients");
   cudaStream_t st = (cudaStream_t)stream;
   const unsigned blk = balanced_block(batch), grid = ceil_div(batch, blk);
+  const unsigned cblk = one_wave_block(batch), cgrid = ceil_div(batch, cblk);
   const double* S = p->sinv;
   const float* S32 = p->sinv32;
   if (refine) {
@@ -401,6 +428,8 @@ extern "C" int penta_cyclic_solve_batched(chx_penta_plan* p, void* rhs, int batc
     else
       penta_per_kernel<float, false><<<pgrid, kPerThreads, 0, st>>>((float*)rhs, nullptr, p->n, batch,
                                                                     (const float*)p->d_fac);
+  } else if (p->d_circ && circ_pays(p->n, p->circ_rows, batch, 5, 4, 8.0)) {
+    penta_circ_kernel<<<cgrid, cblk, 0, st>>>((double*)rhs, p->n, batch, p->d_circ, p->circ_rows);
   } else if (p->dtype == CHX_F64) {
     double* x = (double*)rhs;
     penta_solve_kernel<double, double, double><<<grid, blk, 0, st>>>(x, x, p->n, batch, (const double*)p->d_fac, S[0],
