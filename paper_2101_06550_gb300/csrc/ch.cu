@@ -238,34 +238,8 @@ __global__ void __launch_bounds__(kT* kRBY, kRLapMinBlocks) ch_rhs_r_kernel(cons
   }
   if constexpr (NOISE == kNoiseDraw) {
     if (d_step) step = *d_step;
-    const uint64_t key1 = sim0 + (uint64_t)z;
-    double* rx = dev + (size_t)z * 2 * N;
-    double* ry = rx + N;
-    constexpr int kPairs = kT / 2 + 1;  // per staged row: the west halo's pair, then the tile's
-    for (int q = tid; q < (kT + 1) * kPairs; q += kT * kRBY) {
-      const int a = q / kPairs, h = q - a * kPairs;
-      const int gj = wrap_near(j0 - 1 + a, ny);
-      const int gi = h == 0 ? (i0 == 0 ? nx : i0) - 2 : i0 + 2 * (h - 1);  // even: first point of the pair
-      if (gi >= nx) continue;                                               // ragged last tile
-      float x0, y0, x1, y1;
-      const size_t p = (size_t)gj * nx + gi;
-      deviate_pair(p >> 1, step, seed, key1, &x0, &y0, &x1, &y1);
-      if (h == 0) {
-        s_dx[a][0] = x1;
-        s_dy[a][0] = y1;
-      } else {
-        s_dx[a][2 * h - 1] = x0;
-        s_dy[a][2 * h - 1] = y0;
-        s_dx[a][2 * h] = x1;
-        s_dy[a][2 * h] = y1;
-        if (a >= 1 && j0 + a - 1 < ny) {  // the tile's own points
-          rx[p] = f2d_exact(x0);
-          rx[p + 1] = f2d_exact(x1);
-          ry[p] = f2d_exact(y0);
-          ry[p + 1] = f2d_exact(y1);
-        }
-      }
-    }
+    stage_deviates<kT, kT * kRBY>(s_dx, s_dy, dev + (size_t)z * 2 * N, nx, ny, i0, j0, tid, step, seed,
+                                  sim0 + (uint64_t)z);
   }
   __syncthreads();
   const size_t ldo = (size_t)G * ny;
@@ -764,6 +738,7 @@ int put_lo(float* dst, const std::vector<double>& src) {
 }
 
 int dir_alloc(SpikeDir* D, int n, int P, int slots) {
+  D->circ_ok.assign(slots, 0);
   D->n = n;
   D->P = P;
   D->m = n / P;
@@ -821,6 +796,12 @@ int dir_set(SpikeDir* D, int z, double a) {
     }
     if (D->phi < D->plo) D->phi = D->plo;
   }
+  if (D->d_circ) {
+    FxDir cd;
+    D->circ_ok[z] = fx_dir_host(D->n, D->cP, D->cm, a, &cd);
+    if (D->circ_ok[z] && (rc = cuda_check(cudaMemcpy(D->d_circ + z, &cd, sizeof(cd), cudaMemcpyHostToDevice), "ch: upload")))
+      return rc;
+  }
   const size_t m4 = 4 * (size_t)D->m, kk = (size_t)16 * D->P * D->P;
   const int P = D->P, K = 4 * P;
   std::vector<double> rb(kk);
@@ -855,6 +836,9 @@ int dir_replicate(SpikeDir* D) {
   int rc = CHX_OK;
   for (int z = 1; z < D->slots && !rc; ++z) {
     rc = cuda_check(cudaMemcpy(D->d_a + z, D->d_a, sizeof(double), cudaMemcpyDeviceToDevice), "ch: replicate");
+    D->circ_ok[z] = D->circ_ok[0];
+    if (!rc && D->d_circ)
+      rc = cuda_check(cudaMemcpy(D->d_circ + z, D->d_circ, sizeof(FxDir), cudaMemcpyDeviceToDevice), "ch: replicate");
     if (!rc) rc = cuda_check(cudaMemcpy(D->d_lu + z * m4, D->d_lu, m4 * 8, cudaMemcpyDeviceToDevice), "ch: replicate");
     if (!rc) rc = cuda_check(cudaMemcpy(D->d_vw + z * m4, D->d_vw, m4 * 8, cudaMemcpyDeviceToDevice), "ch: replicate");
     if (!rc) rc = cuda_check(cudaMemcpy(D->d_rinv + z * kk, D->d_rinv, kk * 8, cudaMemcpyDeviceToDevice), "ch: replicate");
@@ -875,12 +859,14 @@ int dir_replicate(SpikeDir* D) {
 
 int dir_move(SpikeDir* D, int from, int to, cudaStream_t st) {
   const size_t m4 = 4 * (size_t)D->m, kk = (size_t)16 * D->P * D->P;
-  struct { void* base; size_t esz, per; } a[15] = {
+  D->circ_ok[to] = D->circ_ok[from];
+  struct { void* base; size_t esz, per; } a[16] = {{D->d_circ, D->d_circ ? sizeof(FxDir) : 0, 1},
       {D->d_a, 8, 1}, {D->d_lu, 8, m4}, {D->d_vw, 8, m4}, {D->d_rinv, 8, kk}, {D->d_a32, 4, 1},
       {D->d_aff, 8, 1}, {D->d_lu4, 4, m4}, {D->d_vw32, 4, m4}, {D->d_rinv32, 4, kk}, {D->d_vwlo, 4, m4},
       {D->d_rinvlo, 4, kk}, {D->d_rb32, 4, kk}, {D->d_rblo, 4, kk}, {D->d_vw4, 4, m4}, {D->d_vw4lo, 4, m4}};
   for (auto& x : a) {
     const size_t b = x.esz * x.per;
+    if (b == 0) continue;
     int rc = cuda_check(cudaMemcpyAsync((char*)x.base + to * b, (char*)x.base + from * b, b, cudaMemcpyDeviceToDevice, st),
                         "ch: move parameters");
     if (rc) return rc;
@@ -893,6 +879,7 @@ void free_dir(SpikeDir* D) {
   cudaFree(D->d_a32); cudaFree(D->d_aff); cudaFree(D->d_lu4); cudaFree(D->d_vw32); cudaFree(D->d_rinv32);
   cudaFree(D->d_vwlo); cudaFree(D->d_rinvlo); cudaFree(D->d_rb32); cudaFree(D->d_rblo);
   cudaFree(D->d_vw4); cudaFree(D->d_vw4lo);
+  cudaFree(D->d_circ);
   *D = SpikeDir();
 }
 
@@ -1028,6 +1015,8 @@ std::vector<int> segment_candidates(int n, int nsys, int precision) {
 
 static int group_move_params_gl(ChGroup* g, int from, int to) {
   int rc = cuda_check(cudaMemcpy(g->d_gl + to, g->d_gl + from, 8, cudaMemcpyDeviceToDevice), "ch: replicate");
+  if (!rc && g->d_fxgl)
+    rc = cuda_check(cudaMemcpy(g->d_fxgl + to, g->d_fxgl + from, sizeof(FxGl), cudaMemcpyDeviceToDevice), "ch: replicate");
   if (!rc) rc = cuda_check(cudaMemcpy(g->d_glff + to, g->d_glff + from, 8, cudaMemcpyDeviceToDevice), "ch: replicate");
   return rc;
 }
@@ -1041,6 +1030,7 @@ static int prepare_kernels() {
   if (rc || dev < 0 || dev >= 64 || done[dev]) return rc;
   balanced_block(0);  // reads the SM count now, outside any stream capture
   rc = prepare_solve_ff();
+  if (!rc) rc = prepare_adi();
   if (!rc) done[dev] = true;
   return rc;
 }
@@ -1072,6 +1062,15 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   g->kff.k1 = split_ff(g->k1);
   g->kff.k2 = split_ff(g->k2);
   int rc;
+  g->fused = precision == CHX_PREC_F64 && adi_shape(nx, ny, G, &g->adi);
+  if (g->fused) {
+    g->X.cP = g->adi.xP, g->X.cm = g->adi.xm;
+    g->Y.cP = g->adi.yP, g->Y.cm = g->adi.ym;
+    if ((rc = dev_alloc(&g->X.d_circ, G)) || (rc = dev_alloc(&g->Y.d_circ, G)) || (rc = dev_alloc(&g->d_fxgl, G))) {
+      group_free(g);
+      return rc;
+    }
+  }
   if ((rc = dir_alloc(&g->X, nx, px ? px : default_segments(nx, G * ny, precision), G)) ||
       (rc = dir_alloc(&g->Y, ny, py ? py : default_segments(ny, nx * G, precision), G)) || (rc = dev_alloc(&g->d_gl, G)) ||
       (rc = dev_alloc(&g->d_glff, G)) || (rc = group_set_gamma(g, 0, gamma)) || (rc = dir_replicate(&g->X)) ||
@@ -1086,9 +1085,9 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   {
     auto dir_bytes = [&](const SpikeDir& D) {
       const size_t m4 = 4 * (size_t)D.m, kk = (size_t)16 * D.P * D.P;
-      return (size_t)G * (8 + 4 + 8 + m4 * (8 + 8 + 4 + 4 + 4 + 4 + 4) + kk * (8 + 4 + 4 + 4 + 4));
+      return (size_t)G * ((D.d_circ ? sizeof(FxDir) : 0) + 8 + 4 + 8 + m4 * (8 + 8 + 4 + 4 + 4 + 4 + 4) + kk * (8 + 4 + 4 + 4 + 4));
     };
-    g->factor_bytes = dir_bytes(g->X) + dir_bytes(g->Y) + (size_t)G * (sizeof(double) + sizeof(float2));
+    g->factor_bytes = dir_bytes(g->X) + dir_bytes(g->Y) + (size_t)G * (sizeof(double) + sizeof(float2) + (g->fused ? sizeof(FxGl) : 0));
   }
   for (int z = 1; z < G && !rc; ++z) rc = group_move_params_gl(g, 0, z);
   if (rc) {
@@ -1133,6 +1132,11 @@ int group_set_gamma(ChGroup* g, int z, double gamma) {
   if ((rc = cuda_check(cudaMemcpy(g->d_gl + z, &gl, sizeof(double), cudaMemcpyHostToDevice), "ch: gamma upload")))
     return rc;
   if (z == 0) g->gamma = gamma;
+  if (g->d_fxgl) {
+    const FxGl fxgl = fx_gl_host(gl, gamma / (g->dy * g->dy));
+    if ((rc = cuda_check(cudaMemcpy(g->d_fxgl + z, &fxgl, sizeof(fxgl), cudaMemcpyHostToDevice), "ch: gamma upload")))
+      return rc;
+  }
   return cuda_check(cudaMemcpy(g->d_glff + z, &glff, sizeof(float2), cudaMemcpyHostToDevice), "ch: gamma upload");
 }
 
@@ -1140,6 +1144,9 @@ int group_move_params(ChGroup* g, int from, int to, cudaStream_t st) {
   if (from == to) return CHX_OK;
   int rc;
   if ((rc = dir_move(&g->X, from, to, st)) || (rc = dir_move(&g->Y, from, to, st))) return rc;
+  if (g->d_fxgl && (rc = cuda_check(cudaMemcpyAsync(g->d_fxgl + to, g->d_fxgl + from, sizeof(FxGl),
+                                                    cudaMemcpyDeviceToDevice, st), "ch: move")))
+    return rc;
   if ((rc = cuda_check(cudaMemcpyAsync(g->d_gl + to, g->d_gl + from, 8, cudaMemcpyDeviceToDevice, st), "ch: move")))
     return rc;
   return cuda_check(cudaMemcpyAsync(g->d_glff + to, g->d_glff + from, 8, cudaMemcpyDeviceToDevice, st), "ch: move");
@@ -1152,6 +1159,8 @@ void group_free(ChGroup* g) {
   free_dir(&g->Y);
   cudaFree(g->d_gl);
   cudaFree(g->d_glff);
+  cudaFree(g->d_fxgl);
+  g->d_fxgl = nullptr;
   g->d_gl = nullptr;
   g->d_glff = nullptr;
 }
@@ -1180,6 +1189,28 @@ static void launch_reduced(const TC* yb, const DirView<TC>& D, TC* tau, int nsys
   const unsigned blk = balanced_block((size_t)nsys * D.P * (4 / R) * Z);
   spike_reducedR_kernel<TC, kReducedRows><<<dim3(ceil_div(nsys, blk), D.P * (4 / R), Z), blk, 0, st>>>(
       yb, D, tau, nsys, ybz, scale);
+}
+
+// The FP64 step in three launches.
+static void step_fused(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
+                    Prof* prof) {
+  const AdiShape& s = g->adi;
+  double* f = wptr<double>(work, g->off_f);
+  const FxRhs R{g->nx, g->ny, G, g->d_fxgl, g->rho, g->k1 / g->k2, f, g->noise, g->noise_w, g->nkx / g->k2,
+                g->nky / g->k2, g->noise_seed, g->noise_sim0, g->noise_step, g->noise_dstep};
+  const AdiStep P{g->nx, g->ny, G, s.xr, s.xP, s.xm, s.ys, s.yP, s.ym, g->X.d_circ, g->Y.d_circ, f,
+                 wptr<long long>(work, g->off_w), wptr<int2>(work, g->off_m), g->k2};
+  { PROF(kRhs); launch_fx_rhs(R, cur, prev, st); }
+  { PROF(kXSolve); launch_adi_x(P, s, st); }
+  { PROF(kYSolve); launch_adi_y(P, s, cur, prev, keep_roles, st); }
+}
+
+// Whether the first G slots' operators all have circulant tables.
+static bool fused_serves(const ChGroup* g, int G) {
+  if (!g->fused) return false;
+  for (int z = 0; z < G; ++z)
+    if (!g->X.circ_ok[z] || !g->Y.circ_ok[z]) return false;
+  return true;
 }
 
 static void step_f64(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
@@ -1253,7 +1284,8 @@ void group_cook_clear(ChGroup* g) {
 
 void group_step(ChGroup* g, int gact, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
                 Prof* prof, int* status) {
-  if (g->precision == CHX_PREC_F64) step_f64(g, gact, cur, prev, work, keep_roles, st, prof, status);
+  if (fused_serves(g, gact)) step_fused(g, gact, cur, prev, work, keep_roles, st, prof);
+  else if (g->precision == CHX_PREC_F64) step_f64(g, gact, cur, prev, work, keep_roles, st, prof, status);
   else step_f32r(g, gact, cur, prev, work, keep_roles, st, prof);
 }
 

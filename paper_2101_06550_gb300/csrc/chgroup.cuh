@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "chx_internal.cuh"
+#include "fx.cuh"
 #include "mixed.cuh"
 
 namespace chx {
@@ -49,6 +50,10 @@ struct SpikeDir {
   bool pset = false;
   // refinement passes of the mixed-precision solves, for the stiffest slot
   int passes = 1;
+  // FP64 groups: the fused solves' tables, cm rows in cP segments, and which slots have one
+  FxDir* d_circ = nullptr;
+  int cP = 0, cm = 0;
+  std::vector<char> circ_ok;
 };
 // Refinement passes for the operator I + a delta^4: one up to a = 5e4 (the
 // 2048^2 workload's a = 1.9e4 meets 1e-6 with one), two above.  Measured at
@@ -161,6 +166,44 @@ int ens_phase_occupancy(int phase, size_t smem);
 // keep the current group's parameters in static shared memory besides).
 size_t ens_phase_smem_max();
 
+// The fused solves of an FP64 step (adi_fx.cu).
+constexpr int kAdiNan = 1 << 30;       // exponent of a block with infinities or NaN
+constexpr int kAdiSmem = 227 * 1024;   // most shared memory of a block
+struct AdiShape {
+  int xr, xP, xm, xnt;   // x solve: rows per block, segments of xm points, threads
+  int ys, yP, ym, ynt;   // y solve: columns per block, segments of ym points, threads
+  size_t xsm, ysm;       // dynamic shared memory
+};
+struct AdiStep {
+  int nx, ny, G;
+  int xr, xP, xm, ys, yP, ym;
+  const FxDir *X, *Y;    // per slot
+  const double* f;       // right-hand side over k2, row major
+  long long* w;          // x solve's result (times kappa_x) and, per block of rows, the exponents
+  int2* wexp;            // of its unit and of its largest value
+  double k2;
+};
+int prepare_adi();
+// Block shapes for G fields of nx x ny; false when a strip does not fit in shared memory.
+bool adi_shape(int nx, int ny, int G, AdiShape* s);
+void launch_adi_x(const AdiStep& P, const AdiShape& s, cudaStream_t st);
+void launch_adi_y(const AdiStep& P, const AdiShape& s, double* cur, double* prev, int keep_roles, cudaStream_t st);
+
+// The fixed-point right-hand side (rhs_fx.cu): r / k2, row major, into f.
+struct FxRhs {
+  int nx, ny, G;
+  const FxGl* gl;        // per slot
+  double rho, kd;        // dx^2 / dy^2, dx^2 / dt
+  double* f;
+  // Cahn-Hilliard-Cook forcing (nkx, nky over k2): deviates given (noise), or drawn into draw
+  const double* noise;
+  double* draw;
+  double nkx, nky;
+  uint64_t seed, sim0, step;
+  const uint64_t* d_step;
+};
+void launch_fx_rhs(const FxRhs& P, const double* cur, const double* prev, cudaStream_t st);
+
 // Per-kernel CUDA-event timing (ch_profile).
 enum ProfSlot { kRhs, kLocX, kRedX, kRefX, kLoc2X, kRed2X, kFinX, kLocY, kRedY, kRefY, kLoc2Y, kRed2Y, kUpd, kRhsLap,
                 kXSolve, kYSolve, kSlots };
@@ -209,10 +252,13 @@ struct ChGroup {
   const uint64_t* noise_dstep = nullptr;
   struct ObsState* obs = nullptr;  // observables scratch, made on first use (obs.cu)
   float2* d_glff = nullptr;
+  FxGl* d_fxgl = nullptr;                    // slots, with fused
   SpikeDir X, Y;
   // work layout (byte offsets), for G fields
   size_t off_f = 0, off_flo = 0, off_w = 0, off_wlo = 0, off_y1 = 0, off_y2 = 0, off_x0 = 0, off_cb = 0, off_m = 0;
   size_t off_ybx = 0, off_tx = 0, off_ybx2 = 0, off_tx2 = 0, off_yby = 0, off_ty = 0, off_yby2 = 0, off_ty2 = 0;
+  bool fused = false;  // FP64: the fused solves' blocks fit (adi); a step takes them when every slot has tables
+  AdiShape adi{};
   size_t work_bytes = 0;
   size_t factor_bytes = 0;  // device bytes of the per-slot factors and parameters (group_init)
 };

@@ -1,5 +1,6 @@
 // Host factorisation of symmetric definite circulant band rows (circulant.cuh).
 #include "circulant.cuh"
+#include "fx.cuh"
 
 #include <math.h>
 
@@ -124,6 +125,135 @@ bool circ_factor_host(int n, double a_, double b_, double c_, double scale, Circ
   for (int j = 0; j < R + 3 && j < n + 3; ++j) t[kCircH + j] = h[j].hi + h[j].lo;
   for (int k = 0; k < (int)out->tab.size(); ++k)
     if (!isfinite(t[k])) return false;
+  return true;
+}
+
+namespace {
+// v as an integer multiple of 2^-62 in two signed halves
+int2 q62(long double v) {
+  const long long k = llroundl(v * 4611686018427387904.0L);
+  const int lo = (int)(uint32_t)k;
+  return make_int2((int)((k - lo) >> 32), lo);
+}
+}  // namespace
+
+FxGl fx_gl_host(double gx, double gy) {
+  FxGl o{make_int2(0, 0), make_int2(0, 0), -100, 0};
+  if (!(gx + gy > 0)) return o;
+  int e = 0;
+  frexp(gx + gy, &e);  // gx + gy < 2^e
+  o.q = e + 1;
+  o.gx = q62(ldexpl((long double)gx, -o.q));
+  o.gy = q62(ldexpl((long double)gy, -o.q));
+  return o;
+}
+
+bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
+  typedef long double ld;
+  if (!(a > 0) || a > kFxStiff) return false;
+  // z + 1 / z = 2 + s with s^2 = -1 / a: the root inside the unit circle and its conjugate give
+  // L = 1 - 2 Re z S^{-1} + |z|^2 S^{-2}.  As multiples of 2^-62: rounded to FP64, they would
+  // move the gains of the smooth modes, whose |L|^2 is 1 / a, by 2^-45.
+  const ld im = 1 / sqrtl((ld)a), wr = -im * im / 4;  // s = i im, w = s + s^2 / 4
+  const ld p = sqrtl(wr * wr + im * im), ri = sqrtl((p - wr) / 2), rr = im / (2 * ri);  // sqrt(w)
+  const ld or_ = 1 + rr, oi = im / 2 + ri, oo = or_ * or_ + oi * oi;                       // 1 / z
+  out->k1 = q62(2 * or_ / oo);
+  out->k2 = q62(-1 / oo);
+  auto fixed = [](int2 k) { return ((long long)k.x << 32) + k.y; };
+  auto as_dd = [](long long k) {
+    dd v;
+    v.hi = (double)k;
+    v.lo = (double)(k - (long long)v.hi) * 0x1p-62;
+    v.hi *= 0x1p-62;
+    return v;
+  };
+  const dd d1 = as_dd(fixed(out->k1)), d2 = as_dd(fixed(out->k2));  // -l1, -l2
+  const double l2 = -d2.hi;
+  const ld at1 = (ld)((1ll << 62) - fixed(out->k1) - fixed(out->k2)) * 0x1p-62L;
+  if (!(at1 > 0) || out->k1.x == 0) return false;  // k1 = 0: nothing but ties to round
+  out->scale = (double)(at1 * at1);                // the mean's gain is 1
+  // h_r = -l1 h_{r-1} - l2 h_{r-2} until it has decayed (h[r + 1] = h_r)
+  std::vector<dd> h(n + 3);
+  dd p1, p2;
+  p1.hi = 1;
+  double most = 0, both = 0, norm = 0;
+  int W = 0;
+  bool decayed = false;
+  for (int r = 0; r < (1 << 16) && !decayed; ++r) {  // p1 = h_r, p2 = h_{r-1}
+    if (r + 1 < n + 3) h[r + 1] = p1;
+    norm += fabs(p1.hi);
+    both = fabs(p1.hi - l2 * p2.hi) > both ? fabs(p1.hi - l2 * p2.hi) : both;
+    most = fabs(p1.hi) > most ? fabs(p1.hi) : most;
+    if (fabs(p1.hi) >= 0x1p-62) W = r + 1;
+    decayed = fabs(p1.hi) < 0x1p-80 && fabs(p2.hi) < 0x1p-80;
+    const dd nx = dd_add(dd_mul2(p1, d1), dd_mul2(p2, d2));
+    p2 = p1;
+    p1 = nx;
+  }
+  if (!decayed || !(norm < 0x1p11)) return false;
+  auto H = [&](int r) { return r < 0 ? 0.0L : (ld)h[r + 1].hi + (ld)h[r + 1].lo; };
+  auto transfer = [&](int len, ld (&t)[4]) {
+    const ld k2 = (ld)d2.hi + d2.lo;
+    t[0] = H(len), t[1] = k2 * H(len - 1), t[2] = H(len - 1), t[3] = len > 1 ? k2 * H(len - 2) : 0.0L;
+  };
+  auto put = [](const ld (&t)[4], int2* o, int q) {
+    for (int k = 0; k < 4; ++k) o[k] = q62(t[k] / (ld)(1 << q));
+  };
+  auto bits = [](const ld (&t)[4]) {
+    ld mx = 0;
+    for (int k = 0; k < 4; ++k) mx = fabsl(t[k]) > mx ? fabsl(t[k]) : mx;
+    int q = 0;
+    while (q < 30 && mx >= (ld)(1 << q)) ++q;
+    return q;
+  };
+  const int llen = n - (P - 1) * m;
+  ld tn[4], cl[4], ts[kFxLevels][2][4] = {};
+  transfer(n, tn);
+  out->qs = 0;
+  for (int k = 0; k < kFxLevels && (1 << k) <= P; ++k)
+    for (int s = 0; s < 2; ++s) {
+      const int len = P == 1 ? n : (1 << k) * m + (s ? llen - m : 0);
+      transfer(len < n ? len : n, ts[k][s]);
+      out->qs = bits(ts[k][s]) > out->qs ? bits(ts[k][s]) : out->qs;
+    }
+  const ld a00 = 1 - tn[0], a11 = 1 - tn[3], det = a00 * a11 - tn[1] * tn[2];
+  if (!(fabsl(det) > 0)) return false;
+  cl[0] = a11 / det, cl[1] = tn[1] / det, cl[2] = tn[2] / det, cl[3] = a00 / det;
+  out->qc = bits(cl);
+  if (out->qs > 6 || out->qc > 6) return false;
+  for (int k = 0; k < kFxLevels; ++k)
+    for (int s = 0; s < 2; ++s) put(ts[k][s], out->step[k][s], out->qs);
+  put(cl, out->close, out->qc);
+  out->W = W + 2;
+  // segments back from which a state is still felt, whichever of them is the short one
+  int J = 1;
+  while (J < P && (J - 1) * m + llen < out->W) ++J;
+  out->J = J;
+  out->L = 0;
+  while ((1 << out->L) < J) ++out->L;
+  if ((1 << out->L) > P || out->L > kFxLevels || J == P) out->L = -1;
+  // growth of a state, and of the sum over J segments (their transfer matrices commute:
+  // powers of the recurrence's), doubled for the way round
+  auto ceil_log2 = [](double v) {
+    int q = 0;
+    while (q < 60 && v > (double)(1ll << q)) ++q;
+    return q;
+  };
+  out->a1 = (float)(1.001 * most);
+  out->a2 = (float)(1.001 * both);
+  double sum = 1;
+  for (int j = 1; j < 2 * J && j < P; ++j) {
+    const int len = j * m < n ? j * m : n;
+    sum += (double)(fabsl(H(len)) + fabsl((ld)l2 * H(len - 1)) + fabsl(H(len - 1)));
+  }
+  if (J == P) {
+    ld mx = 0;
+    for (int k = 0; k < 4; ++k) mx = fabsl(cl[k]) > mx ? fabsl(cl[k]) : mx;
+    sum *= 1 + 2 * (double)mx;
+  }
+  const int eb = ceil_log2(2 * sum) - 4;  // states below 2^55 may sum to 2^59
+  out->eb = eb > 0 ? eb : 0;
+  if (most > 64 || out->eb > 6) return false;  // with the norm: shifts below 32
   return true;
 }
 

@@ -9,6 +9,8 @@
 #pragma once
 #include <stdint.h>
 
+#include "ff.cuh"
+
 namespace chx {
 
 __device__ __forceinline__ void philox4x64_10(uint64_t& x0, uint64_t& x1, uint64_t& x2, uint64_t& x3, uint64_t k0,
@@ -48,6 +50,43 @@ __device__ __forceinline__ void deviate_pair(uint64_t b, uint64_t step, uint64_t
   philox4x64_10(w0, w1, w2, w3, seed, sim);
   box_muller(w0, w1, x0, y0);
   box_muller(w2, w3, x1, y1);
+}
+
+// Draws the deviates of the T x T tile at (i0, j0) and of the column before and the
+// row above it into s_dx and s_dy ([a][b] is grid point (i0 - 1 + b, j0 - 1 + a),
+// wrapped), and stores the tile's own to rho (planes rho^x, rho^y of nx * ny) as they
+// are drawn.  nx even, so that a pair never straddles rows.  NT threads, thread tid.
+template <int T, int NT>
+__device__ __forceinline__ void stage_deviates(float (*s_dx)[T + 1], float (*s_dy)[T + 1], double* rho, int nx, int ny,
+                                               int i0, int j0, int tid, uint64_t step, uint64_t seed, uint64_t sim) {
+  double* rx = rho;
+  double* ry = rho + (size_t)nx * ny;
+  constexpr int kPairs = T / 2 + 1;  // per staged row: the west halo's pair, then the tile's
+  for (int q = tid; q < (T + 1) * kPairs; q += NT) {
+    const int a = q / kPairs, h = q - a * kPairs;
+    int gj = j0 - 1 + a;
+    gj = gj < 0 ? gj + ny : gj % ny;
+    const int gi = h == 0 ? (i0 == 0 ? nx : i0) - 2 : i0 + 2 * (h - 1);  // even: first point of the pair
+    if (gi >= nx) continue;                                               // ragged last tile
+    float x0, y0, x1, y1;
+    const size_t p = (size_t)gj * nx + gi;
+    deviate_pair(p >> 1, step, seed, sim, &x0, &y0, &x1, &y1);
+    if (h == 0) {
+      s_dx[a][0] = x1;
+      s_dy[a][0] = y1;
+    } else {
+      s_dx[a][2 * h - 1] = x0;
+      s_dy[a][2 * h - 1] = y0;
+      s_dx[a][2 * h] = x1;
+      s_dy[a][2 * h] = y1;
+      if (a >= 1 && j0 + a - 1 < ny) {  // the tile's own points
+        rx[p] = f2d_exact(x0);
+        rx[p + 1] = f2d_exact(x1);
+        ry[p] = f2d_exact(y0);
+        ry[p + 1] = f2d_exact(y1);
+      }
+    }
+  }
 }
 
 }  // namespace chx
