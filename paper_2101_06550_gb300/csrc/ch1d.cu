@@ -217,7 +217,7 @@ extern "C" int ch1d_step(chx_ch1d_plan* p, double* c, int nsteps, void* stream) 
   cudaStream_t st = (cudaStream_t)stream;
   const unsigned blk = balanced_block(p->batch), grid = ceil_div(p->batch, blk);
   const unsigned cblk = one_wave_block(p->batch), cgrid = ceil_div(p->batch, cblk);
-  const bool circ = p->d_circ && circ_pays(p->n, p->circ_rows, p->batch, 10, 4, 14.0);
+  const bool circ = p->d_circ && circ_pays(p->n, p->circ_rows, p->batch, 10, 4, 13.0);
   for (int k = 0; k < nsteps; ++k) {
     if (circ)
       ch1d_circ_kernel<<<cgrid, cblk, 0, st>>>(c, p->n, p->batch, p->d_circ, p->circ_rows);

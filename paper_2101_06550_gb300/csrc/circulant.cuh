@@ -56,7 +56,9 @@ bool circ_factor_host(int n, double a, double b, double c, double scale, CircTab
 // 107 -> 72 us).  With more it is the operation count, against lu_ops per row of
 // the LU form: its 9 or 5 operations issue a little closer together, so the
 // solves pass 8 and 4.5 here (pentadiagonal 98 x 197152 at R = 0.9 n, 8.6
-// operations: 335 us against 315), the time steps their LU forms' 14, 10 and 6.
+// operations: 335 us against 315), the 1D Cahn-Hilliard step 13 (14 operations in its LU
+// form; 64 x 332992 and 111 x 420704 at R = n: 591 and 1225 us against 544 and 1154), the
+// Crank-Nicolson steps their LU forms' 10 and 6.
 bool circ_pays(int n, int R, int batch, int ops, int closure_ops, double lu_ops);
 // Uploads a table into *dst (cudaMalloc).
 int circ_upload(const CircTable& t, double** dst, const char* what);
