@@ -115,41 +115,13 @@ __device__ __forceinline__ void fx_sweep(long long* p, int st, int cnt, int2 k1,
   for (; cnt > 0; --cnt, p += st) row(*p, p);
 }
 
-// The state entering segment seg of a system by Horner's rule, from the states e its segments leave
-// when entered with zero: e[q * es], e[q * es + eo].  dir = -1: from the segments
-// below (forward sweep), +1: from those above.
-__device__ __forceinline__ FxState fx_enter(const FxDir& D, const long long* e, int es, int eo, int P, int seg,
-                                            int dir) {
-  FxState s;
-  int q = seg + dir * D.J;
-  if (q < 0) q += P;
-  if (q >= P) q -= P;
-  for (int j = D.J; j > 0; --j) {
-    const int2* T = D.step[0][q == P - 1];
-    const FxVal a = fx_halves(s.g1), b = fx_halves(s.g2);
-    const long long e1 = e[q * es], e2 = e[q * es + eo];
-    s.g1 = fx_dot2(e1, T[0], a, T[1], b, D.qs);
-    s.g2 = fx_dot2(e2, T[2], a, T[3], b, D.qs);
-    q -= dir;
-    if (q < 0) q = P - 1;
-    if (q >= P) q = 0;
-  }
-  if (D.J == P) {  // all the way round
-    const FxVal a = fx_halves(s.g1), b = fx_halves(s.g2);
-    s.g1 = fx_dot2(0, D.close[0], a, D.close[1], b, D.qc);
-    s.g2 = fx_dot2(0, D.close[2], a, D.close[3], b, D.qc);
-  }
-  return s;
-}
-
 // Shared words besides the points: the slot's table, the maximum of the loaded
-// values' high words (x) or the exponent of the strip (y), the shifts of the two
+// values' high words (x), the shifts of the two
 // sweeps and the bits of their results' high words, the place of the block's sweepers;
 // then the segments' states.
 struct FxShared {
   FxDir D;
   unsigned maxhi;
-  int top, bad;
   int shift[4], big[2], turn;
 };
 
@@ -164,8 +136,7 @@ __device__ __forceinline__ void fx_begin(FxShared* sh, const FxDir* d, int sweep
     ((long long*)&sh->D)[k] = ((const long long*)d)[k];
   if (threadIdx.x == 0) {
     sh->maxhi = 0;
-    sh->top = -(1 << 20);
-    sh->bad = sh->big[0] = sh->big[1] = 0;
+    sh->big[0] = sh->big[1] = 0;
     for (int k = 0; k < 4; ++k) sh->shift[k] = k & 1 ? -64 : 0;
     unsigned w;
     asm("mov.u32 %0, %%warpid;" : "=r"(w));
@@ -206,35 +177,62 @@ __device__ __forceinline__ int fx_half(FxShared* sh, int* shift, int* big, int t
   }
   __syncthreads();
   int over = -64;
-  if (D.L >= 0) {  // the states of 1, 2, 4, ... segments before this one, two buffers in turn
-    auto from = [&](int k) {  // the segment k before this one
-      int q = seg + dir * k;
-      q += q < 0 ? P : q >= P ? -P : 0;
-      return (q - seg) * es;
-    };
-    if (mine) {
-      s.g1 = e[from(1)];
-      s.g2 = e[from(1) + eo];
-    }
-    for (int l = 0; l < D.L; ++l) {
-      const int k = 1 << l, buf = l & 1 ? 0 : 2 * eo;
+  // The state entering the segment, from those that the `count` before it leave when
+  // entered with zero: those of 1, 2, 4, ... in two buffers in turn, summed by count's bits
+  // (300 rows of a stiff operator in 60 segments: 12 steps, where Horner's rule takes 60).
+  auto from = [&](int k) {  // the segment k before this one
+    int q = seg + dir * k;
+    q += q < 0 ? P : q >= P ? -P : 0;
+    return (q - seg) * es;
+  };
+  // whether the last segment is among the k before this one
+  auto last = [&](int k) { return dir < 0 ? seg < k : k == P || (seg < P - 1 && seg + k >= P - 1); };
+  auto across = [&](const int2 (&M)[2][4], int k, int buf, FxState& v) {
+    const int o = buf + from(k);
+    const FxVal a = fx_halves(e[o]), b = fx_halves(e[o + eo]);
+    const int2* T = M[last(k)];
+    v.g1 = fx_dot2(v.g1, T[0], a, T[1], b, D.qs);
+    v.g2 = fx_dot2(v.g2, T[2], a, T[3], b, D.qs);
+  };
+  FxState a;
+  if (mine) {
+    a.g1 = e[from(1)];
+    a.g2 = e[from(1) + eo];
+  }
+  if ((D.count & (D.count - 1)) == 0) {
+    for (int l = 0; D.count >> (l + 1); ++l) {
+      const int buf = l & 1 ? 0 : 2 * eo;
       if (mine) {
-        e[buf] = s.g1;
-        e[buf + eo] = s.g2;
+        e[buf] = a.g1;
+        e[buf + eo] = a.g2;
       }
       __syncthreads();
-      if (mine) {
-        const int o = buf + from(k);
-        const FxVal a = fx_halves(e[o]), b = fx_halves(e[o + eo]);
-        const int2* M = D.step[l][dir < 0 ? seg < k : seg < P - 1 && seg + k >= P - 1];
-        s.g1 = fx_dot2(s.g1, M[0], a, M[1], b, D.qs);
-        s.g2 = fx_dot2(s.g2, M[2], a, M[3], b, D.qs);
-      }
+      if (mine) across(D.step[l], 1 << l, buf, a);
     }
-  } else if (mine) {
-    s = fx_enter(D, e - seg * es, es, eo, P, seg, dir);
+    s = a;
+  } else {
+    int have = 0;  // segments in s
+    for (int l = 0; D.count >> l; ++l) {
+      const int buf = l & 1 ? 0 : 2 * eo;
+      if (mine) {
+        e[buf] = a.g1;
+        e[buf + eo] = a.g2;
+      }
+      __syncthreads();
+      if (D.count >> l & 1) {
+        if (mine && have) across(D.rest[l], have, buf, s);
+        else s = a;
+        have += 1 << l;
+      }
+      if (mine && D.count >> (l + 1)) across(D.step[l], 1 << l, buf, a);
+    }
   }
   if (mine) {
+    if (D.round) {
+      const FxVal u = fx_halves(s.g1), v = fx_halves(s.g2);
+      s.g1 = fx_dot2(0, D.close[0], u, D.close[1], v, D.qc);
+      s.g2 = fx_dot2(0, D.close[2], u, D.close[3], v, D.qc);
+    }
     // |g| <= the probe's + |h_{r+1} g1 - l2 h_r g2|, the latter with g1 = g2 + (g1 - g2)
     const float local = (float)(mag + 1) / (float)(1 << up);
     const float bound = local + D.a2 * (float)(fx_mag(s.g2) + 2) + D.a1 * (float)(fx_mag(s.g1 - s.g2) + 2);
@@ -322,9 +320,8 @@ __global__ void __launch_bounds__(NT) adi_x_kernel(AdiStep P) {
   if ((threadIdx.x & 31) == 0) atomicMax(&sh->maxhi, m);
   __syncthreads();
   const unsigned mh = sh->maxhi;
-  int2* ex = P.wexp + (size_t)z * gridDim.x + blockIdx.x;
   if (mh >= 0x7ff00000u) {  // infinities or NaN: no solution
-    if (threadIdx.x == 0) *ex = make_int2(0, kAdiNan);
+    if (threadIdx.x == 0) atomicMax(&P.wtop[z], kAdiNan);
     return;
   }
   const int E = fx_exponent(mh);
@@ -349,7 +346,8 @@ __global__ void __launch_bounds__(NT) adi_x_kernel(AdiStep P) {
   }
   if (threadIdx.x == 0) {  // the results' unit 2^S, and the exponent of the largest
     const int S = E - 1076 + t;
-    *ex = make_int2(S, S + 32 + sh->big[1]);
+    P.wunit[(size_t)z * gridDim.x + blockIdx.x] = S;
+    atomicMax(&P.wtop[z], S + 32 + sh->big[1]);
   }
 }
 
@@ -371,30 +369,17 @@ __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double
   const int eo = S * P.yP;
   long long* x = e + 4 * eo;
   const int ms = y_pitch(S, P.ym);
-  signed char* shift = (signed char*)(x + ms * P.yP);  // per block of rows of the x solve
   const size_t base = (size_t)z * n * P.nx + col0;
   const long long* __restrict__ w = P.w + base;
   cn += base;
   cp += base;
   fx_begin(sh, P.Y + z, eo);
   __syncthreads();
-  // one exponent for the strip: its largest value takes 54 bits
-  const int nex = (n + P.xr - 1) / P.xr;
-  const int2* __restrict__ ex = P.wexp + (size_t)z * nex;
-  int top = -(1 << 20), bad = 0;
-  for (int k = threadIdx.x; k < nex; k += NT) {
-    const int v = ex[k].y;
-    bad |= v == kAdiNan;
-    top = max(top, v);
-  }
-  top = __reduce_max_sync(0xffffffffu, top);
-  if ((threadIdx.x & 31) == 0) atomicMax(&sh->top, top);
-  if (bad) sh->bad = 1;
-  __syncthreads();
-  const bool finite = !sh->bad;
-  const int unit = sh->top - 54;
-  for (int k = threadIdx.x; k < nex; k += NT) shift[k] = (signed char)max(-64, min(unit - ex[k].x, 63));
-  __syncthreads();
+  // one exponent for the strip: the field's largest value takes 54 bits
+  const int top = P.wtop[z];
+  const bool finite = top != kAdiNan;
+  const int unit = top - 54;
+  const int* __restrict__ units = P.wunit + (size_t)z * ((n + P.xr - 1) / P.xr);
   const int dj = NT / S, j0 = threadIdx.x / S, i = threadIdx.x - j0 * S;
   const bool in = i < cols;
   const size_t dp = (size_t)dj * P.nx;
@@ -404,7 +389,7 @@ __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double
     Walk k(j0, dj, P.ym, S, ms);
 #pragma unroll 8
     for (; k.j < n; k.next(), p += dp) {
-      const int d = shift[P.xr == 1 ? k.j : (int)__umulhi((unsigned)k.j, rx)];
+      const int d = max(-63, min(unit - units[P.xr == 1 ? k.j : (int)__umulhi((unsigned)k.j, rx)], 63));
       long long v = in && finite ? *p : 0;
       if (d < 0) v <<= -d;
       if (d >= 32) v = fx_shift(v >> 32, d - 32);
@@ -427,7 +412,7 @@ __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double
     }
   const int len = seg == P.yP - 1 ? n - seg * P.ym : P.ym;
   const int t = fx_solve<false>(sh, mine, x + seg * ms + sys, S, len, e + tid, S, eo, P.yP, seg);
-  const double c = scalbn(P.k2 * sh->D.scale * P.X[z].scale, unit + t);
+  const double c = P.k2 * sh->D.scale * P.X[z].scale;
   if (!in) return;
   size_t p = (size_t)j0 * P.nx + i;
   for (Walk k(j0, dj, P.ym, S, ms); k.j < n; p += kUpd * dp) {
@@ -446,7 +431,7 @@ __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double
 #pragma unroll
     for (int u = 0; u < kUpd; ++u)
       if (u < left) {
-        double v = fma(c, (double)x[o[u]], fma(2.0, a[u], -b[u]));
+        double v = fma(c, fx_to_double(x[o[u]], unit + t), fma(2.0, a[u], -b[u]));
         if (!finite) v = __longlong_as_double(0x7ff8000000000000ll);
         if (keep_roles) {
           cp[p + u * dp] = a[u];
@@ -459,9 +444,7 @@ __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double
 }
 
 size_t adi_bytes(int states, size_t points) { return 8 * ((size_t)kHead + 4 * (size_t)states + points); }
-size_t adi_y_bytes(int S, int P, int n, int xr) {
-  return adi_bytes(S * P, (size_t)P * y_pitch(S, (n + P - 1) / P)) + (((size_t)n / xr + 8) & ~(size_t)7);
-}
+size_t adi_y_bytes(int S, int P, int n) { return adi_bytes(S * P, (size_t)P * y_pitch(S, (n + P - 1) / P)); }
 
 int segments(int n, int most) {
   int P = n / 8 < most ? n / 8 : most;
@@ -505,7 +488,7 @@ bool adi_shape(int nx, int ny, int G, AdiShape* s) {
   s->ynt = (size_t)ny * S >= 1024 ? 512 : 256;
   s->yP = segments(ny, 64);
   s->ym = (ny + s->yP - 1) / s->yP;
-  s->ysm = adi_y_bytes(S, s->yP, ny, s->xr);
+  s->ysm = adi_y_bytes(S, s->yP, ny);
   return s->ysm <= (size_t)kAdiSmem;
 }
 

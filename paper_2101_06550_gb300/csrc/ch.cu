@@ -1036,7 +1036,7 @@ static int prepare_kernels() {
 }
 
 int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, double dt, int precision, int G,
-               int px, int py) {
+               int px, int py, bool single) {
   if (int rc0 = prepare_kernels()) return rc0;
   if (nx < 8 || ny < 8 || nx > 16384 || ny > 16384)
     return fail(CHX_EINVAL, "ch: nx %d, ny %d outside [8, 16384]", nx, ny);
@@ -1062,7 +1062,12 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   g->kff.k1 = split_ff(g->k1);
   g->kff.k2 = split_ff(g->k2);
   int rc;
-  g->fused = precision == CHX_PREC_F64 && adi_shape(nx, ny, G, &g->adi);
+  // The fixed-point step also serves an FP32+refine plan, more accurately, where it is the
+  // faster one: up to 2^20 points and sides of 1400 (us per step, FP32+refine against
+  // fixed point: 128^2 68, 22; 512^2 46, 33; 1024^2 69, 64; 777 x 1311 106, 72; but 1280^2
+  // 90, 100; 2048 x 300 53, 79; 2048^2 161, 180).
+  const bool refine = single && (size_t)nx * ny <= 1u << 20 && nx <= 1400 && ny <= 1400;
+  g->fused = (precision == CHX_PREC_F64 || refine) && adi_shape(nx, ny, G, &g->adi);
   if (g->fused) {
     g->X.cP = g->adi.xP, g->X.cm = g->adi.xm;
     g->Y.cP = g->adi.yP, g->Y.cm = g->adi.ym;
@@ -1191,15 +1196,17 @@ static void launch_reduced(const TC* yb, const DirView<TC>& D, TC* tau, int nsys
       yb, D, tau, nsys, ybz, scale);
 }
 
-// The FP64 step in three launches.
+// The step in fixed-point arithmetic (fx.cuh): three launches.  FP32+refine groups have
+// the same space in the pairs of FP32 arrays of r and w.
 static void step_fused(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
                     Prof* prof) {
   const AdiShape& s = g->adi;
   double* f = wptr<double>(work, g->off_f);
-  const FxRhs R{g->nx, g->ny, G, g->d_fxgl, g->rho, g->k1 / g->k2, f, g->noise, g->noise_w, g->nkx / g->k2,
+  int* wtop = wptr<int>(work, g->off_cb);  // G, then the units
+  const FxRhs R{g->nx, g->ny, G, g->d_fxgl, g->rho, g->k1 / g->k2, f, wtop, g->noise, g->noise_w, g->nkx / g->k2,
                 g->nky / g->k2, g->noise_seed, g->noise_sim0, g->noise_step, g->noise_dstep};
   const AdiStep P{g->nx, g->ny, G, s.xr, s.xP, s.xm, s.ys, s.yP, s.ym, g->X.d_circ, g->Y.d_circ, f,
-                 wptr<long long>(work, g->off_w), wptr<int2>(work, g->off_m), g->k2};
+                 wptr<long long>(work, g->off_w), wtop + G, wtop, g->k2};
   { PROF(kRhs); launch_fx_rhs(R, cur, prev, st); }
   { PROF(kXSolve); launch_adi_x(P, s, st); }
   { PROF(kYSolve); launch_adi_y(P, s, cur, prev, keep_roles, st); }
@@ -1262,7 +1269,7 @@ static void step_f32r(ChGroup* g, int G, double* cur, double* prev, void* work, 
 
 int group_cook_deviates(ChGroup* g, int gact, double* rho, uint64_t seed, uint64_t sim0, uint64_t step,
                         const uint64_t* d_step, cudaStream_t st) {
-  if (g->precision == CHX_PREC_F64 && g->nx % 2 == 0) {
+  if ((g->precision == CHX_PREC_F64 || fused_serves(g, gact)) && g->nx % 2 == 0) {
     g->noise = nullptr;
     g->noise_w = rho;
     g->noise_seed = seed;
@@ -1321,7 +1328,7 @@ extern "C" int ch_plan_create(chx_ch_plan** plan, int nx, int ny, double lx, dou
   new (&p->g) ChGroup();
   p->prof = new Prof();
   int rc = hdr_init(&p->hdr, kMagicCh);
-  if (!rc) rc = group_init(&p->g, nx, ny, lx, ly, gamma, dt, precision, 1);
+  if (!rc) rc = group_init(&p->g, nx, ny, lx, ly, gamma, dt, precision, 1, 0, 0, true);
   if (rc) { ch_plan_free(p); return rc; }
   if (cudaMalloc(&p->d_partials, 3 * (size_t)kDiagBlocks * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();

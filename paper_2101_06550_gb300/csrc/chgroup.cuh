@@ -50,7 +50,7 @@ struct SpikeDir {
   bool pset = false;
   // refinement passes of the mixed-precision solves, for the stiffest slot
   int passes = 1;
-  // FP64 groups: the fused solves' tables, cm rows in cP segments, and which slots have one
+  // groups with fused solves: their tables, cm rows in cP segments, and which slots have one
   FxDir* d_circ = nullptr;
   int cP = 0, cm = 0;
   std::vector<char> circ_ok;
@@ -179,8 +179,8 @@ struct AdiStep {
   int xr, xP, xm, ys, yP, ym;
   const FxDir *X, *Y;    // per slot
   const double* f;       // right-hand side over k2, row major
-  long long* w;          // x solve's result (times kappa_x) and, per block of rows, the exponents
-  int2* wexp;            // of its unit and of its largest value
+  long long* w;          // x solve's result (times kappa_x), in units 2^wunit per block of rows,
+  int *wunit, *wtop;     // below 2^wtop for each simulation (set by the right-hand side first)
   double k2;
 };
 int prepare_adi();
@@ -195,6 +195,7 @@ struct FxRhs {
   const FxGl* gl;        // per slot
   double rho, kd;        // dx^2 / dy^2, dx^2 / dt
   double* f;
+  int* wtop;             // AdiStep's, reset here
   // Cahn-Hilliard-Cook forcing (nkx, nky over k2): deviates given (noise), or drawn into draw
   const double* noise;
   double* draw;
@@ -257,7 +258,7 @@ struct ChGroup {
   // work layout (byte offsets), for G fields
   size_t off_f = 0, off_flo = 0, off_w = 0, off_wlo = 0, off_y1 = 0, off_y2 = 0, off_x0 = 0, off_cb = 0, off_m = 0;
   size_t off_ybx = 0, off_tx = 0, off_ybx2 = 0, off_tx2 = 0, off_yby = 0, off_ty = 0, off_yby2 = 0, off_ty2 = 0;
-  bool fused = false;  // FP64: the fused solves' blocks fit (adi); a step takes them when every slot has tables
+  bool fused = false;  // the fused solves' blocks fit (adi); a step takes them when every slot has tables
   AdiShape adi{};
   size_t work_bytes = 0;
   size_t factor_bytes = 0;  // device bytes of the per-slot factors and parameters (group_init)
@@ -265,9 +266,9 @@ struct ChGroup {
 
 // Validates, factorises both directions on the host (FP64) for `gamma` and
 // uploads them into every slot.  px / py > 0 force the segment counts (the
-// ensemble autotuner); 0 = default.
+// ensemble autotuner); 0 = default.  single: a plan's group (stepped by group_step).
 int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, double dt, int precision, int G,
-               int px = 0, int py = 0);
+               int px = 0, int py = 0, bool single = false);
 // Refactorises slot z of the group for a new gamma (host FP64, synchronous upload).
 int group_set_gamma(ChGroup* g, int z, double gamma);
 // Sets up the Cahn-Hilliard-Cook deviates of the group's next step for its

@@ -209,12 +209,27 @@ bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
   const int llen = n - (P - 1) * m;
   ld tn[4], cl[4], ts[kFxLevels][2][4] = {};
   transfer(n, tn);
+  // segments back from which a state is still felt, whichever of them is the short one;
+  // a power of two where there are as many
+  out->W = W + 2;
+  int J = 1;
+  while (J < P && (J - 1) * m + llen < out->W) ++J;
+  out->round = J == P;
+  int pow2 = 1;
+  while (pow2 < J) pow2 *= 2;
+  out->count = !out->round && pow2 <= P ? pow2 : J;
+  ld rs[kFxLevels][2][4] = {};
   out->qs = 0;
-  for (int k = 0; k < kFxLevels && (1 << k) <= P; ++k)
+  for (int k = 0; k < kFxLevels && (1 << k) <= out->count; ++k)
     for (int s = 0; s < 2; ++s) {
-      const int len = P == 1 ? n : (1 << k) * m + (s ? llen - m : 0);
-      transfer(len < n ? len : n, ts[k][s]);
-      out->qs = bits(ts[k][s]) > out->qs ? bits(ts[k][s]) : out->qs;
+      auto over = [&](int segs, ld (&t)[4]) {
+        const int len = segs * m + (s ? llen - m : 0);
+        transfer(len < n ? len : n, t);
+        out->qs = bits(t) > out->qs ? bits(t) : out->qs;
+      };
+      over(1 << k, ts[k][s]);
+      const int low = out->count & ((1 << k) - 1);
+      if (low) over(low, rs[k][s]);
     }
   const ld a00 = 1 - tn[0], a11 = 1 - tn[3], det = a00 * a11 - tn[1] * tn[2];
   if (!(fabsl(det) > 0)) return false;
@@ -222,16 +237,11 @@ bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
   out->qc = bits(cl);
   if (out->qs > 6 || out->qc > 6) return false;
   for (int k = 0; k < kFxLevels; ++k)
-    for (int s = 0; s < 2; ++s) put(ts[k][s], out->step[k][s], out->qs);
+    for (int s = 0; s < 2; ++s) {
+      put(ts[k][s], out->step[k][s], out->qs);
+      put(rs[k][s], out->rest[k][s], out->qs);
+    }
   put(cl, out->close, out->qc);
-  out->W = W + 2;
-  // segments back from which a state is still felt, whichever of them is the short one
-  int J = 1;
-  while (J < P && (J - 1) * m + llen < out->W) ++J;
-  out->J = J;
-  out->L = 0;
-  while ((1 << out->L) < J) ++out->L;
-  if ((1 << out->L) > P || out->L > kFxLevels || J == P) out->L = -1;
   // growth of a state, and of the sum over J segments (their transfer matrices commute:
   // powers of the recurrence's), doubled for the way round
   auto ceil_log2 = [](double v) {

@@ -25,13 +25,13 @@ constexpr int kFxLevels = 7;  // up to 128 segments
 struct FxDir {
   int2 k1, k2;          // -l1, -l2
   // state transfer over 2^k segments, and over as many with the last (short) one among
-  // them, / 2^qs
-  int2 step[kFxLevels][2][4];
+  // them, / 2^qs; the same over the segments of the lower bits of `count`
+  int2 step[kFxLevels][2][4], rest[kFxLevels][2][4];
   int2 close[4];        // (1 - transfer over the system)^{-1}, / 2^qc
   int qs, qc;
   int W;                // rows after which a state has decayed below 2^-62
-  int J;                // segments a state reaches (P: all, through `close`)
-  int L;                // J <= 2^L <= P, or -1
+  int count;            // segments put together: as many as a state reaches, or all P of them
+  int round;            // (through `close`)
   int eb;               // bits the sum over segments of the states they leave can grow by
   // |h_{r+1} g1 - l2 h_r g2| <= a1 |g1 - g2| + a2 |g2|
   float a1, a2;
@@ -133,6 +133,21 @@ __device__ __forceinline__ long long fx_shift(long long f, int t) {
   f += (unsigned)((1u << t) >> 1) - any + odd;
   return (long long)(((unsigned long long)(unsigned)((int)(f >> 32) >> t) << 32) |
                      __funnelshift_r((unsigned)f, (unsigned)(f >> 32), t));
+}
+
+// x 2^S as FP64, rounded to nearest (0 and infinity outside its range).  24 integer
+// instructions where a conversion instruction takes the FP64 unit for 64 cycles per warp.
+__device__ __forceinline__ double fx_to_double(long long x, int S) {
+  const long long s = x >> 63;
+  const unsigned long long a = (unsigned long long)((x ^ s) - s);
+  const int lz = __clzll((long long)a);
+  const unsigned long long n = a << (lz & 63);
+  const int e = 1023 + 63 - lz + S;
+  unsigned long long b = (n >> 11) + ((n >> 10) & 1);  // 53 bits, or 2^53
+  b += (unsigned long long)(unsigned)(e - 1) << 52;
+  if (a == 0 || e <= 0) b = 0;
+  if (e >= 2047) b = 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
 }
 
 // High word of |g|, within one unit.
