@@ -28,7 +28,7 @@
 namespace chx {
 namespace {
 
-constexpr int kU = 7;    // rows loaded ahead in the sweeps
+constexpr int kU = 8;    // rows loaded ahead in the sweeps
 constexpr int kUpd = 4;  // points of the update loaded ahead
 
 struct FxState {
@@ -37,12 +37,12 @@ struct FxState {
 
 // Rows p, p + st, ... (cnt of them) from state zero, for the state they leave, in a unit
 // 2^t times the values' own.  At first |f| <= 2^53 in it; when a state passes 2^55 after a
-// block of kU rows, the thread goes over to a coarser one (the state below 2^55 again).  The first
-// kU + 1 rows cannot take it to 2^60: a unit impulse grows to 9 and the sum of eight to
-// 36 at most.  mag: the largest high word (at most twice it), in the last unit.
+// block of kU rows, the thread goes over to a coarser one (the state below 2^55 again).  Eight
+// rows cannot take it to 2^60: a state grows to 9 + 8 times itself and the sum of eight
+// values to 36 at most.  mag: the largest high word (at most twice it), in the last unit.
 __device__ __forceinline__ void fx_probe(const long long* p, int st, int cnt, int2 k1, int2 k2, FxState& s, int& t,
                                          int& mag) {
-  static_assert(kU <= 7, "growth within a block of rows");
+  static_assert(kU <= 8, "growth within a block of rows");
   long long g1 = 0, g2 = 0;
   FxVal v1{0, 0}, v2{0, 0};
   int mx = 0, m = 0, up = 1 << (30 - t);
@@ -70,11 +70,27 @@ __device__ __forceinline__ void fx_probe(const long long* p, int st, int cnt, in
   };
   // the first row is f alone, whose ties fx_step would round up: fx_shift keeps the odd
   // symmetry of the step
-  g1 = fx_shift(*p, t);
-  v1 = fx_halves(g1);
-  m = fx_mag(g1);
-  p += st;
-  for (--cnt; cnt >= kU; cnt -= kU) {
+  auto first = [&](long long f) {
+    g1 = fx_shift(f, t);
+    v1 = fx_halves(g1);
+    m = fx_mag(g1);
+  };
+  if (cnt >= kU) {
+    long long b[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) b[u] = p[u * st];
+    first(b[0]);
+#pragma unroll
+    for (int u = 1; u < kU; ++u) row(b[u]);
+    cnt -= kU;
+    p += kU * st;
+    check();
+  } else {
+    first(*p);
+    p += st;
+    --cnt;
+  }
+  for (; cnt >= kU; cnt -= kU) {
     long long b[kU];
 #pragma unroll
     for (int u = 0; u < kU; ++u) b[u] = p[u * st];
@@ -83,6 +99,7 @@ __device__ __forceinline__ void fx_probe(const long long* p, int st, int cnt, in
     p += kU * st;
     check();
   }
+#pragma unroll 1
   for (; cnt > 0; --cnt, p += st) row(*p);
   check();
   s.g1 = g1;
@@ -112,6 +129,7 @@ __device__ __forceinline__ void fx_sweep(long long* p, int st, int cnt, int2 k1,
     for (int u = 0; u < kU; ++u) row(b[u], p + u * st);
     p += kU * st;
   }
+#pragma unroll 1
   for (; cnt > 0; --cnt, p += st) row(*p, p);
 }
 
