@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "chx_internal.cuh"
+#include "circ_fx.cuh"
 #include "circulant.cuh"
 
 using namespace chx;
@@ -29,6 +30,9 @@ struct chx_ch1d_plan {
   double sinv[4];
   double* d_circ;  // circulant table, [13] alpha (nullptr when sigma is beyond it and the LU factors serve)
   int circ_rows;
+  CircFx* d_fx;  // its fixed-point form (nullptr: the range does not serve)
+  int2 fx_alpha;  // alpha / 2^qa < 1/2
+  int fx_qa;
 };
 
 namespace {
@@ -154,6 +158,57 @@ __global__ void __launch_bounds__(kMaxBlockWarps * 32) ch1d_circ_kernel(double* 
       [](int) { return 0.0; }, [&](int r, double y, double) { pc[(size_t)r * B] = y * sc; });
 }
 
+// The same in fixed point (circ_fx.cuh), after a pass over the system for its largest value:
+// C in units of 2^(e1 - 56), |C| < 2^e1; C (C^2 - 1) as in the 2D right-hand side (rhs_fx.cu).
+// The integer pipes take a row in about 300 cycles per warp and scheduler, the FP64 unit its
+// 10 to 14 operations in 670 to 940: 256 x 262144 on a GB300 1608 -> 825 us, 64 x 332992 545 ->
+// 263 us, 64 x 2048 44 -> 31 us; errors 1.8e-14 -> 6e-15 (2-norm, 256 x 262144).
+__global__ void __launch_bounds__(128) ch1d_fx_kernel(double* c, int n, int batch, const CircFx* __restrict__ tab,
+                                                      int2 alpha, int qa) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= batch) return;
+  const size_t B = (size_t)batch;
+  double* pc = c + s;
+  const int E = fx_column_exponent(pc, B, n);
+  if (E == 2047) {
+    for (int r = 0; r < n; ++r) pc[(size_t)r * B] = __longlong_as_double(0x7ff8000000000000ll);
+    return;
+  }
+  const int e1 = E - 1022, e2 = e1 > 0 ? e1 : 0;
+  const int sl = e1 > -2 ? 3 + 2 * (e1 - e2) : 0, sr = sl > 0 ? 0 : min(-3 - 2 * (e1 - e2), 63);
+  const long long one = e2 <= 31 ? 1ll << (62 - 2 * e2) : 0;
+  // |f| <= |C| + 4 alpha |N| < 2^eb; C and alpha N to its unit by 2^-t1 and 2^-t2
+  const int hb = tab->hb, un = e1 + 2 * e2 - 59 + qa;
+  const int uf = max(e1, e1 + 2 * e2 + qa + 1) + 1 - 59 + hb;
+  int t1 = uf - (e1 - 56), t2 = uf - un;
+  const int pre1 = t1 > 30 ? min(t1 - 30, 63) : 0, pre2 = t2 > 30 ? min(t2 - 30, 63) : 0;
+  const int u1 = 1 << (30 - min(t1, 30)), u2 = 1 << (30 - min(t2, 30));
+  const int2 k1 = tab->k1, k2 = tab->k2;
+  auto nl = [&](long long v) {
+    const FxVal kc = fx_halves(v << 6), gc = fx_halves(v << 3);
+    const FxVal ku = fx_halves(((fx_mul(make_int2(kc.h, kc.l), gc) << sl) >> sr) - one);
+    return fx_mul(make_int2(ku.h, ku.l), gc);
+  };
+  const double c0 = pc[0];
+  long long ccur = fx_from_double(c0, E, 56), Ncur = nl(ccur);
+  long long Nprev = nl(fx_from_double(pc[(size_t)(n - 1) * B], E, 56));
+  const double sc = tab->scale;
+  const int S = uf + hb;
+  circ_fx_sweeps(
+      n, tab, (long long*)pc, B,
+      [&](int r) { return r + 1 < n ? pc[(size_t)(r + 1) * B] : c0; },  // C_{r+1}; row 0 is overwritten by then
+      [&](double cn1, FxVal v1, FxVal v2) {
+        const long long cn = fx_from_double(cn1, E, 56), Nn = nl(cn);
+        const long long an = fx_mul(alpha, fx_halves(Nn - 2 * Ncur + Nprev));
+        const long long g = fx_step2(fx_halves(ccur >> pre1), u1, fx_halves(an >> pre2), u2, k1, v1, k2, v2);
+        Nprev = Ncur;
+        Ncur = Nn;
+        ccur = cn;
+        return g;
+      },
+      [](int) { return 0.0; }, [&](int r, long long y, double) { pc[(size_t)r * B] = fx_to_double(y, S) * sc; });
+}
+
 }  // namespace
 
 namespace chx {
@@ -161,6 +216,7 @@ void ch1d_plan_free(chx_ch1d_plan* p) {
   if (!p) return;
   if (p->d_fac) cudaFree(p->d_fac);
   if (p->d_circ) cudaFree(p->d_circ);
+  if (p->d_fx) cudaFree(p->d_fx);
   hdr_free(&p->hdr);
   free(p);
 }
@@ -205,6 +261,14 @@ extern "C" int ch1d_plan_create(chx_ch1d_plan** plan, int n, int batch, double l
     ct.tab[13] = p->alpha;
     p->circ_rows = ct.R;
     rc = circ_upload(ct, &p->d_circ, "ch1d_plan_create");
+    CircFx fx;
+    std::vector<int2> h;
+    if (!rc && circ_fx_host(n, sigma, 1.0, &fx, &h)) {
+      rc = circ_fx_upload(fx, h, &p->d_fx, "ch1d_plan_create");
+      const FxGl al = fx_gl_host(p->alpha, 0.0);  // alpha / 2^qa, below 1/2
+      p->fx_alpha = al.gx;
+      p->fx_qa = al.q;
+    }
   }
   if (rc) { ch1d_plan_free(p); return rc; }
   *plan = p;
@@ -217,9 +281,12 @@ extern "C" int ch1d_step(chx_ch1d_plan* p, double* c, int nsteps, void* stream) 
   cudaStream_t st = (cudaStream_t)stream;
   const unsigned blk = balanced_block(p->batch), grid = ceil_div(p->batch, blk);
   const unsigned cblk = one_wave_block(p->batch), cgrid = ceil_div(p->batch, cblk);
+  const unsigned fblk = balanced_block(p->batch) < 128 ? balanced_block(p->batch) : 128;
   const bool circ = p->d_circ && circ_pays(p->n, p->circ_rows, p->batch, 10, 4, 13.0);
   for (int k = 0; k < nsteps; ++k) {
-    if (circ)
+    if (p->d_fx)
+      ch1d_fx_kernel<<<ceil_div(p->batch, fblk), fblk, 0, st>>>(c, p->n, p->batch, p->d_fx, p->fx_alpha, p->fx_qa);
+    else if (circ)
       ch1d_circ_kernel<<<cgrid, cblk, 0, st>>>(c, p->n, p->batch, p->d_circ, p->circ_rows);
     else
       ch1d_step_kernel<<<grid, blk, 0, st>>>(c, p->n, p->batch, p->alpha, p->d_fac, p->sinv[0], p->sinv[1],

@@ -1,5 +1,6 @@
 // Host factorisation of symmetric definite circulant band rows (circulant.cuh).
 #include "circulant.cuh"
+#include "circ_fx.cuh"
 #include "fx.cuh"
 
 #include <math.h>
@@ -148,17 +149,25 @@ FxGl fx_gl_host(double gx, double gy) {
   return o;
 }
 
-bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
+namespace {
+// 1 + a delta^4 = kappa L L^T with -l1, -l2 multiples of 2^-62.
+struct Biharmonic {
+  int2 k1, k2;   // -l1, -l2
+  dd d1, d2;
+  double scale;  // 1 / kappa
+};
+
+// z + 1 / z = 2 + s with s^2 = -1 / a: the root inside the unit circle and its conjugate give
+// L = 1 - 2 Re z S^{-1} + |z|^2 S^{-2}.  Rounded to FP64, its coefficients would move the
+// gains of the smooth modes, whose |L|^2 is 1 / a, by 2^-45 at a = 2e4.
+bool factor_biharmonic(double a, Biharmonic* o) {
   typedef long double ld;
-  if (!(a > 0) || a > kFxStiff) return false;
-  // z + 1 / z = 2 + s with s^2 = -1 / a: the root inside the unit circle and its conjugate give
-  // L = 1 - 2 Re z S^{-1} + |z|^2 S^{-2}.  As multiples of 2^-62: rounded to FP64, they would
-  // move the gains of the smooth modes, whose |L|^2 is 1 / a, by 2^-45.
+  if (!(a > 0) || !isfinite(a)) return false;
   const ld im = 1 / sqrtl((ld)a), wr = -im * im / 4;  // s = i im, w = s + s^2 / 4
   const ld p = sqrtl(wr * wr + im * im), ri = sqrtl((p - wr) / 2), rr = im / (2 * ri);  // sqrt(w)
-  const ld or_ = 1 + rr, oi = im / 2 + ri, oo = or_ * or_ + oi * oi;                       // 1 / z
-  out->k1 = q62(2 * or_ / oo);
-  out->k2 = q62(-1 / oo);
+  const ld zr = 1 + rr, zi = im / 2 + ri, zz = zr * zr + zi * zi;                          // 1 / z
+  o->k1 = q62(2 * zr / zz);
+  o->k2 = q62(-1 / zz);
   auto fixed = [](int2 k) { return ((long long)k.x << 32) + k.y; };
   auto as_dd = [](long long k) {
     dd v;
@@ -167,11 +176,24 @@ bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
     v.hi *= 0x1p-62;
     return v;
   };
-  const dd d1 = as_dd(fixed(out->k1)), d2 = as_dd(fixed(out->k2));  // -l1, -l2
+  o->d1 = as_dd(fixed(o->k1));
+  o->d2 = as_dd(fixed(o->k2));
+  const ld at1 = (ld)((1ll << 62) - fixed(o->k1) - fixed(o->k2)) * 0x1p-62L;
+  if (!(at1 > 0x1p-14L) || o->k1.x == 0) return false;  // k1 = 0: nothing but ties to round
+  o->scale = (double)(at1 * at1);                       // the mean's gain is 1
+  return true;
+}
+}  // namespace
+
+bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
+  typedef long double ld;
+  Biharmonic F;
+  if (a > kFxStiff || !factor_biharmonic(a, &F)) return false;
+  out->k1 = F.k1;
+  out->k2 = F.k2;
+  out->scale = F.scale;
+  const dd d1 = F.d1, d2 = F.d2;
   const double l2 = -d2.hi;
-  const ld at1 = (ld)((1ll << 62) - fixed(out->k1) - fixed(out->k2)) * 0x1p-62L;
-  if (!(at1 > 0) || out->k1.x == 0) return false;  // k1 = 0: nothing but ties to round
-  out->scale = (double)(at1 * at1);                // the mean's gain is 1
   // h_r = -l1 h_{r-1} - l2 h_{r-2} until it has decayed (h[r + 1] = h_r)
   std::vector<dd> h(n + 3);
   dd p1, p2;
@@ -265,6 +287,82 @@ bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
   out->eb = eb > 0 ? eb : 0;
   if (most > 64 || out->eb > 6) return false;  // with the norm: shifts below 32
   return true;
+}
+
+bool circ_fx_host(int n, double a, double scale, CircFx* out, std::vector<int2>* table) {
+  typedef long double ld;
+  Biharmonic F;
+  if (n < 3 || !factor_biharmonic(a, &F)) return false;
+  // h[r + 1] = h_r until it has decayed, and its 1-norm
+  std::vector<dd> h(n + 3);
+  dd p1, p2;
+  p1.hi = 1;
+  double norm = 0;
+  bool decayed = false;
+  for (int r = 0; r < (1 << 16) && !decayed; ++r) {
+    if (r + 1 < n + 3) h[r + 1] = p1;
+    norm += fabs(p1.hi);
+    decayed = fabs(p1.hi) < 0x1p-100 && fabs(p2.hi) < 0x1p-100;
+    const dd nx = dd_add(dd_mul2(p1, F.d1), dd_mul2(p2, F.d2));
+    p2 = p1;
+    p1 = nx;
+  }
+  if (!decayed || !(norm < 0x1p12)) return false;
+  int hb = 2, R = n;
+  while (1.001 * norm > (double)(1 << hb)) ++hb;
+  while (R > 0 && fabs(h[R].hi) < 0x1p-62 && fabs(h[R + 1].hi) < 0x1p-62) --R;
+  R = (R + kCircU) / kCircU * kCircU;
+  if (R > n) R = n;
+  auto H = [&](int j) { return (ld)h[j].hi + (ld)h[j].lo; };
+  // the closure as in circ_factor_host
+  const ld k2 = (ld)F.d2.hi + F.d2.lo;  // -l2
+  const ld p00 = 1 - H(n + 1), p01 = -k2 * H(n), p10 = -H(n), p11 = 1 - k2 * H(n - 1), det = p00 * p11 - p01 * p10;
+  if (!(fabsl(det) > 0)) return false;
+  const ld A[4] = {p11 / det, -p01 / det, -p10 / det, p00 / det};
+  ld q01 = 0, q00 = 0, qm0 = 0, qm1 = 0;
+  for (int r = 0; r < n && r <= R; ++r) {
+    q01 += H(r + 1) * H(r + 2);
+    q00 += H(r + 1) * H(r + 1);
+    qm0 += H(r) * H(r + 1);
+    qm1 += H(r) * H(r + 2);
+  }
+  const ld M[4] = {q01, k2 * q00, qm1, k2 * qm0};
+  ld AM[4] = {A[0] * M[0] + A[1] * M[2], A[0] * M[1] + A[1] * M[3], A[2] * M[0] + A[3] * M[2],
+              A[2] * M[1] + A[3] * M[3]};
+  ld ma = 0, mm = 0;
+  for (int k = 0; k < 4; ++k) {
+    AM[k] = ldexpl(AM[k], -hb);
+    ma = fabsl(A[k]) > ma ? fabsl(A[k]) : ma;
+    mm = fabsl(AM[k]) > mm ? fabsl(AM[k]) : mm;
+  }
+  out->qc = out->qm = 0;
+  while (out->qc < 20 && ma >= (ld)(1 << out->qc)) ++out->qc;
+  while (out->qm < 20 && mm >= (ld)(1 << out->qm)) ++out->qm;
+  if (out->qc > 1 || out->qm > 8) return false;
+  out->k1 = F.k1;
+  out->k2 = F.k2;
+  for (int k = 0; k < 4; ++k) {
+    out->close[k] = q62(ldexpl(A[k], -out->qc));
+    out->closeM[k] = q62(ldexpl(AM[k], -out->qm));
+  }
+  out->hb = hb;
+  out->R = R;
+  out->scale = F.scale * scale;
+  table->assign(R + 3, make_int2(0, 0));
+  for (int j = 0; j < R + 3 && j < n + 3; ++j) (*table)[j] = q62(ldexpl(H(j), -hb));
+  return true;
+}
+
+int circ_fx_upload(const CircFx& c, const std::vector<int2>& h, CircFx** dst, const char* what) {
+  const size_t hbytes = h.size() * sizeof(int2);
+  if (cudaMalloc(dst, sizeof(CircFx) + hbytes) != cudaSuccess) {
+    cudaGetLastError();
+    *dst = nullptr;
+    return fail(CHX_ENOMEM, "%s: fixed-point table allocation", what);
+  }
+  int rc = cuda_check(cudaMemcpy(*dst, &c, sizeof(CircFx), cudaMemcpyHostToDevice), what);
+  if (!rc) rc = cuda_check(cudaMemcpy(*dst + 1, h.data(), hbytes, cudaMemcpyHostToDevice), what);
+  return rc;
 }
 
 int circ_upload(const CircTable& t, double** dst, const char* what) {

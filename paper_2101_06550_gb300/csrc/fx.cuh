@@ -90,6 +90,21 @@ __device__ __forceinline__ long long fx_step(long long f, int up, int2 k1, FxVal
   return (p << 2) + (c >> 30);
 }
 
+// a 2^-ta + b 2^-tb + k1 g1 + k2 g2, ua = 2^(30 - ta), ub = 2^(30 - tb), rounded once.
+__device__ __forceinline__ long long fx_step2(FxVal a, int ua, FxVal b, int ub, int2 k1, FxVal g1, int2 k2, FxVal g2) {
+  long long c = fx_wide(ua, a.l, 1ll << 29);
+  long long p = fx_wide(ua, a.h, 0);
+  c = fx_wide(ub, b.l, c);
+  p = fx_wide(ub, b.h, p);
+  c = fx_wide(k2.y, g2.h, c);
+  c = fx_wide(k2.x, g2.l, c);
+  p = fx_wide(k2.x, g2.h, p);
+  c = fx_wide(k1.x, g1.l, c);
+  c = fx_wide(k1.y, g1.h, c);
+  p = fx_wide(k1.x, g1.h, p);
+  return (p << 2) + (c >> 30);
+}
+
 // f + (k1 g1 + k2 g2) 2^q to half a unit, 0 <= q < 30, |k1| + |k2| <= 2: low products and
 // the bits below the unit are kept until the scaling.
 __device__ __forceinline__ long long fx_dot2(long long f, int2 k1, FxVal g1, int2 k2, FxVal g2, int q) {
