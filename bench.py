@@ -39,19 +39,17 @@ PREWARM_S = 1.5  # untimed steps before the first measurement (see measure())
 # kernels from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum).
 # ncu flushes the caches before each kernel it measures, so these are cold-cache
 # figures: intermediates that a live step finds in L2 are counted as DRAM reads.
-STEP_DRAM_BYTES_F64 = 373.58e6 + 53.25e6
+STEP_DRAM_BYTES_F64 = 201.63e6 + 11.54e6  # the fixed-point step's three kernels, buffer roles swapped
 STEP_DRAM_BYTES_F32R = 213.10e6 + 63.37e6  # the three fused kernels
 # DRAM bytes (read + write) per launch of the FP64 step's kernels on this
-# workload, from one ncu capture of the current kernels (dram__bytes_read.sum +
-# dram__bytes_write.sum, mean of 3 launches).  The first right-hand-side pass
-# (ch_rhs: Cbar and M) writes two fields that partly stay in L2 for the
-# kernels that read them next.  None: not captured for the current kernel.
-KERNEL_TRAFFIC_BYTES = {"ch_rhs": 67.21e6 + 22.66e6, "ch_rhs_lap": 100.72e6 + 7.47e6}
-# Algorithmic FP64 operations and bytes per grid point of each FP64 kernel.
-KERNEL_FP64_OPS = {"ch_rhs": 8.0, "ch_rhs_lap": 6.0, "spike_local_x": 5.0, "spike_local_y": 5.0, "ch_xfinish": 4.0,
-                   "ch_update": 5.0}
-KERNEL_BYTES = {"ch_rhs": 32, "ch_rhs_lap": 32, "spike_local_x": 16, "spike_local_y": 16, "ch_xfinish": 16,
-                "ch_update": 24}
+# workload, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum).
+KERNEL_TRAFFIC_BYTES = {"ch_rhs": 67.26e6 + 8.61e6, "x_solve_ff": 33.62e6, "y_solve_ff": 100.75e6 + 2.93e6}
+# FP64-pipe operations and algorithmic bytes per grid point of the FP64 step's
+# kernels (its stencils and solves run in fixed point on the integer pipes): the
+# right-hand side reads both fields and writes r, the x solve reads r and writes w,
+# the y solve reads w and both fields and writes both (a one-step call keeps the roles).
+KERNEL_FP64_OPS = {"ch_rhs": 4.0, "x_solve_ff": 0.0, "y_solve_ff": 2.0}
+KERNEL_BYTES = {"ch_rhs": 24, "x_solve_ff": 16, "y_solve_ff": 40}
 
 
 def _peaks():
@@ -190,7 +188,7 @@ def hbm_fraction(pts, ms64, ms32, peak_gbs):
     """The step's HBM traffic against the measured copy bandwidth.  The minimum a
     step must move is 24 B per point (Cn and Cn-1 in, Cn+1 out); the ncu figure
     is every kernel's DRAM bytes, cold-cache.  Both fall far below the peak: the
-    step is bound by the FP64 pipe (the roofline object), not by HBM."""
+    steps are bound by instruction issue and latency, not by HBM."""
     def one(ms, dram):
         d = {"ms_per_step": ms, "algorithmic_bytes_per_step": 24 * pts, "dram_bytes_per_step_ncu_cold": dram,
              "gbs_algorithmic": 24 * pts / (ms * 1e-3) / 1e9,
@@ -392,21 +390,21 @@ def run_chx(args, rank, world, local_rank):
     pts = N * N
     value = world * pts * args.steps / (ms64 * 1e-3)
     peaks = _peaks()
-    # dominant kernel of the FP64 step and its roofline (FP64-pipe bound)
+    # dominant kernel of the FP64 step against the measured copy bandwidth (it is bound
+    # by integer issue and latency; this is its fraction of the memory roofline)
     dom, (dom_ms, dom_n) = max(prof64.items(), key=lambda kv: kv[1][0])
     per_launch_ms = dom_ms / max(1, dom_n)
+    peak = peaks.get("hbm_gbs") or 6800.0
     # the FP64 pipe's rate measured in this process (DFMA throughput kernel, G DP-ops/s)
     fp64_peak_gops = chx.fp64_fma_rate()
-    if dom in KERNEL_FP64_OPS:
-        ach = KERNEL_FP64_OPS[dom] * pts / (per_launch_ms * 1e-3) / 1e9
-        roof = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": fp64_peak_gops, "unit": "G fp64-op/s",
-                "frac": ach / fp64_peak_gops, "fp64_ops_per_point": KERNEL_FP64_OPS[dom],
-                "traffic": KERNEL_TRAFFIC_BYTES.get(dom), "traffic_unit": "bytes per launch",
-                "algorithmic_bytes": KERNEL_BYTES[dom] * pts, "ms_per_launch": per_launch_ms,
-                "peak_source": "in-run chx_fp64_fma_rate (DFMA throughput kernel, same process)"}
-    else:
-        roof = {"kernel": dom, "bound": "alu", "achieved": None, "peak": fp64_peak_gops, "unit": "G fp64-op/s",
-                "frac": None, "traffic": None, "ms_per_launch": per_launch_ms}
+    roof = {"kernel": dom, "bound": "hbm", "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
+            "traffic": KERNEL_TRAFFIC_BYTES.get(dom), "traffic_unit": "bytes per launch", "ms_per_launch": per_launch_ms,
+            "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy bandwidth)" if peaks.get("hbm_gbs") else "fallback",
+            "fp64_fma_rate_gops": fp64_peak_gops}
+    if dom in KERNEL_BYTES:
+        ach = KERNEL_BYTES[dom] * pts / (per_launch_ms * 1e-3) / 1e9
+        roof.update(achieved=ach, frac=ach / peak, algorithmic_bytes=KERNEL_BYTES[dom] * pts,
+                    fp64_ops_per_point=KERNEL_FP64_OPS[dom])
     extras = {}
     if not args.no_extras:
         extras["fp32_refine_accuracy"] = fp32_accuracy(dev)

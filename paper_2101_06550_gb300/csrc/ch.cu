@@ -754,6 +754,14 @@ int dir_alloc(SpikeDir* D, int n, int P, int slots) {
   return CHX_OK;
 }
 
+// Slot z's circulant table for `a`, where there is one (circ_ok).
+int dir_set_circ(SpikeDir* D, int z, double a) {
+  FxDir cd;
+  D->circ_ok[z] = fx_dir_host(D->n, D->cP, D->cm, a, &cd);
+  return D->circ_ok[z] ? cuda_check(cudaMemcpy(D->d_circ + z, &cd, sizeof(cd), cudaMemcpyHostToDevice), "ch: upload")
+                       : CHX_OK;
+}
+
 // Factorises for `a` and uploads into slot z.
 int dir_set(SpikeDir* D, int z, double a) {
   std::vector<double> lu, vw, rinv;
@@ -796,12 +804,7 @@ int dir_set(SpikeDir* D, int z, double a) {
     }
     if (D->phi < D->plo) D->phi = D->plo;
   }
-  if (D->d_circ) {
-    FxDir cd;
-    D->circ_ok[z] = fx_dir_host(D->n, D->cP, D->cm, a, &cd);
-    if (D->circ_ok[z] && (rc = cuda_check(cudaMemcpy(D->d_circ + z, &cd, sizeof(cd), cudaMemcpyHostToDevice), "ch: upload")))
-      return rc;
-  }
+  if (D->d_circ && (rc = dir_set_circ(D, z, a))) return rc;
   const size_t m4 = 4 * (size_t)D->m, kk = (size_t)16 * D->P * D->P;
   const int P = D->P, K = 4 * P;
   std::vector<double> rb(kk);
@@ -1066,6 +1069,7 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   // faster one: up to 2^20 points and sides of 1400 (us per step, FP32+refine against
   // fixed point: 128^2 68, 22; 512^2 46, 33; 1024^2 69, 64; 777 x 1311 106, 72; but 1280^2
   // 90, 100; 2048 x 300 53, 79; 2048^2 161, 180).
+  g->single = single;
   const bool refine = single && (size_t)nx * ny <= 1u << 20 && nx <= 1400 && ny <= 1400;
   g->fused = (precision == CHX_PREC_F64 || refine) && adi_shape(nx, ny, G, &g->adi);
   if (g->fused) {
@@ -1131,7 +1135,13 @@ int group_set_gamma(ChGroup* g, int z, double gamma) {
   const double ax = (2.0 / 3.0) * gamma * g->dt / (g->dx * g->dx * g->dx * g->dx);
   const double ay = (2.0 / 3.0) * gamma * g->dt / (g->dy * g->dy * g->dy * g->dy);
   int rc;
-  if ((rc = dir_set(&g->X, z, ax)) || (rc = dir_set(&g->Y, z, ay))) return rc;
+  // a single plan whose operators both have circulant tables needs no LU factors
+  bool lu = true;
+  if (g->single && g->fused) {
+    if ((rc = dir_set_circ(&g->X, z, ax)) || (rc = dir_set_circ(&g->Y, z, ay))) return rc;
+    lu = !g->X.circ_ok[z] || !g->Y.circ_ok[z];
+  }
+  if (lu && ((rc = dir_set(&g->X, z, ax)) || (rc = dir_set(&g->Y, z, ay)))) return rc;
   const double gl = gamma / (g->dx * g->dx);
   const float2 glff = split_ff(gl);
   if ((rc = cuda_check(cudaMemcpy(g->d_gl + z, &gl, sizeof(double), cudaMemcpyHostToDevice), "ch: gamma upload")))

@@ -237,6 +237,17 @@ extern "C" int ch1d_plan_create(chx_ch1d_plan** plan, int n, int batch, double l
   p->n = n;
   p->batch = batch;
   p->alpha = dt / (dx * dx);
+  CircFx fx;
+  std::vector<int2> h;
+  if (circ_fx_host(n, sigma, 1.0, &fx, &h)) {  // the other forms' tables are not needed then
+    const FxGl al = fx_gl_host(p->alpha, 0.0);  // alpha / 2^qa, below 1/2
+    p->fx_alpha = al.gx;
+    p->fx_qa = al.q;
+    rc = circ_fx_upload(fx, h, &p->d_fx, "ch1d_plan_create");
+    if (rc) { ch1d_plan_free(p); return rc; }
+    *plan = p;
+    return CHX_OK;
+  }
   const double co[5] = {sigma, -4.0 * sigma, 1.0 + 6.0 * sigma, -4.0 * sigma, sigma};
   std::vector<double> rows(5 * (size_t)n);
   for (int k = 0; k < 5; ++k)
@@ -261,14 +272,6 @@ extern "C" int ch1d_plan_create(chx_ch1d_plan** plan, int n, int batch, double l
     ct.tab[13] = p->alpha;
     p->circ_rows = ct.R;
     rc = circ_upload(ct, &p->d_circ, "ch1d_plan_create");
-    CircFx fx;
-    std::vector<int2> h;
-    if (!rc && circ_fx_host(n, sigma, 1.0, &fx, &h)) {
-      rc = circ_fx_upload(fx, h, &p->d_fx, "ch1d_plan_create");
-      const FxGl al = fx_gl_host(p->alpha, 0.0);  // alpha / 2^qa, below 1/2
-      p->fx_alpha = al.gx;
-      p->fx_qa = al.q;
-    }
   }
   if (rc) { ch1d_plan_free(p); return rc; }
   *plan = p;

@@ -258,6 +258,7 @@ struct ChGroup {
   // work layout (byte offsets), for G fields
   size_t off_f = 0, off_flo = 0, off_w = 0, off_wlo = 0, off_y1 = 0, off_y2 = 0, off_x0 = 0, off_cb = 0, off_m = 0;
   size_t off_ybx = 0, off_tx = 0, off_ybx2 = 0, off_tx2 = 0, off_yby = 0, off_ty = 0, off_yby2 = 0, off_ty2 = 0;
+  bool single = false;  // a plan's group: its gamma never changes
   bool fused = false;  // the fused solves' blocks fit (adi); a step takes them when every slot has tables
   AdiShape adi{};
   size_t work_bytes = 0;

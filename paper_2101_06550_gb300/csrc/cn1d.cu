@@ -369,6 +369,14 @@ extern "C" int cn1d_plan_create(chx_cn1d_plan** plan, int order, int n, int batc
     *plan = p;
     return CHX_OK;
   }
+  CircFx fx;
+  std::vector<int2> h;
+  if (order == 4 && circ_fx_host(n, p->sigma, 2.0, &fx, &h)) {  // the other forms' tables are not needed then
+    rc = circ_fx_upload(fx, h, &p->d_fx, "cn1d_plan_create");
+    if (rc) { cn1d_plan_free(p); return rc; }
+    *plan = p;
+    return CHX_OK;
+  }
   std::vector<double> rows(5 * (size_t)n);
   for (int k = 0; k < 5; ++k)
     for (int i = 0; i < n; ++i) rows[(size_t)k * n + i] = v[k];
@@ -401,9 +409,6 @@ extern "C" int cn1d_plan_create(chx_cn1d_plan** plan, int order, int n, int batc
   if (!rc && circ_factor_host(n, order == 4 ? v[0] : 0.0, order == 4 ? v[1] : v[0], order == 4 ? v[2] : v[1], 2.0, &ct)) {
     p->circ_rows = ct.R;
     rc = circ_upload(ct, &p->d_circ, "cn1d_plan_create");
-    CircFx fx;
-    std::vector<int2> h;
-    if (!rc && order == 4 && circ_fx_host(n, p->sigma, 2.0, &fx, &h)) rc = circ_fx_upload(fx, h, &p->d_fx, "cn1d_plan_create");
   }
   if (rc) { cn1d_plan_free(p); return rc; }
   *plan = p;
