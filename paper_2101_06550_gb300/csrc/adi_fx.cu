@@ -10,14 +10,14 @@
 // one exponent (the largest value of the block), and cuts each into P segments, a
 // thread per segment.  A sweep goes over a segment twice: from a zero state for the
 // state it leaves behind, and, once each thread has put together its own starting
-// state from those of the segments before it (Horner's rule with the transfer matrix
-// of a segment), from that state, in place.  So no spikes, reduced systems or
+// state from those of the segments before it (in log2 steps, with the transfer matrices
+// over 1, 2, 4, ... of them), from that state, in place.  So no spikes, reduced systems or
 // corrections: 4 fixed-point steps of two multiply-adds per point and direction.
 //
 // What bounds it: the sweeps' chains (54 cycles per row, six wide multiply-adds on the FMA
 // pipe's half rate and ten other instructions) with one thread per segment, since shared
 // memory holds only 14 rows of 2048 per SM; between them, loads and conversions.  2048^2 on
-// a GB300: 52 us along x, 88 along y with the update.  The LU segment sweeps, reduced solve
+// a GB300: 53 us along x, 81 along y with the update.  The LU segment sweeps, reduced solve
 // and spike corrections that it replaces, three launches per direction and 10.4 FP64
 // operations per point at 2 per clock and SM, took 96 and 103 us; the same two kernels with
 // FP64 sweeps (8.9 operations) 99 and 123.  At 600 x 450 and 128^2 the launches count:
@@ -375,8 +375,8 @@ inline __host__ __device__ int y_pitch(int S, int m) { return m * S + (S <= 8 ? 
 
 // A strip of S columns per block (a power of two), rows S apart in shared memory; a thread
 // stays on one column, NT / S rows from one element to the next.  keep_roles as in
-// group_step.  While the first warps sweep, the others bring the strip of C^n and
-// C^{n-1} into L2 for the update.
+// group_step.  (Bringing the strip of C^n and C^{n-1} into L2 from the idle warps during the
+// sweeps made it slower, 84 against 81 us.)
 template <int NT>
 __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double* cp, int keep_roles) {
   extern __shared__ long long sm[];
@@ -419,15 +419,6 @@ __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double
   const int tid = (threadIdx.x + NT - sh->turn % NT) % NT;
   const int seg = tid / S, sys = tid - seg * S;
   const bool mine = seg < P.yP;
-  const int idle = NT - ((eo + 31) & ~31);  // threads of the warps with nothing to sweep
-  if (tid >= NT - idle)
-    for (int j = tid - (NT - idle); j < n; j += idle) {
-      const double *a = cn + (size_t)j * P.nx, *b = cp + (size_t)j * P.nx;
-      for (int c = 0; c < cols; c += 4) {  // sectors of 32 bytes
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(a + c));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(b + c));
-      }
-    }
   const int len = seg == P.yP - 1 ? n - seg * P.ym : P.ym;
   const int t = fx_solve<false>(sh, mine, x + seg * ms + sys, S, len, e + tid, S, eo, P.yP, seg);
   const double c = P.k2 * sh->D.scale * P.X[z].scale;
@@ -500,7 +491,7 @@ bool adi_shape(int nx, int ny, int G, AdiShape* s) {
   s->xsm = adi_bytes(R * s->xP, (size_t)R * s->xP * (s->xm | 1));
   if (s->xsm > (size_t)kAdiSmem) return false;
   // y: strips of 4 columns, a sector of 32 bytes per row (2048^2: 88 us, 120 us with 2, 100
-  // with 8), of 2 where those are few
+  // with 8, before the last steps), of 2 where those are few
   const int S = (size_t)nx * G >= 512 ? 4 : 2;
   s->ys = S;
   s->ynt = (size_t)ny * S >= 1024 ? 512 : 256;

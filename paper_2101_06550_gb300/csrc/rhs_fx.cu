@@ -23,6 +23,7 @@ namespace chx {
 namespace {
 
 constexpr int kT = 32, kNT = 256;
+constexpr int kBlocks = 5;  // per SM: 49 us at 2048^2, 51 with 4, 6 or 7 (fewer registers)
 constexpr int kB = 56;  // bits of the tile's largest value
 enum : int { kNone, kRead, kDraw };
 
@@ -33,7 +34,7 @@ __device__ __forceinline__ int wrap(int i, int n) {
 }
 
 template <bool kIso, int NOISE>
-__global__ void __launch_bounds__(kNT, 6) fx_rhs_kernel(FxRhs P, const double* __restrict__ cn,
+__global__ void __launch_bounds__(kNT, kBlocks) fx_rhs_kernel(FxRhs P, const double* __restrict__ cn,
                                                         const double* __restrict__ cp) {
   constexpr int kW = kT + 4, kR = kT + 2;
   __shared__ long long s_b[kW][kW + 1];  // Cbar
