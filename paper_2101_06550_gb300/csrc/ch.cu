@@ -1222,11 +1222,12 @@ static void step_fused(ChGroup* g, int G, double* cur, double* prev, void* work,
   { PROF(kYSolve); launch_adi_y(P, s, cur, prev, keep_roles, st); }
 }
 
+bool group_slot_fixed(const ChGroup* g, int z) { return g->fused && g->X.circ_ok[z] && g->Y.circ_ok[z]; }
+
 // Whether the first G slots' operators all have circulant tables.
 static bool fused_serves(const ChGroup* g, int G) {
-  if (!g->fused) return false;
   for (int z = 0; z < G; ++z)
-    if (!g->X.circ_ok[z] || !g->Y.circ_ok[z]) return false;
+    if (!group_slot_fixed(g, z)) return false;
   return true;
 }
 

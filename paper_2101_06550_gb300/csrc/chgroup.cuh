@@ -272,6 +272,9 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
                int px = 0, int py = 0, bool single = false);
 // Refactorises slot z of the group for a new gamma (host FP64, synchronous upload).
 int group_set_gamma(ChGroup* g, int z, double gamma);
+// Whether slot z steps in fixed point: the host picks the launches by it, so a captured graph is
+// good only while no active slot's answer changes.
+bool group_slot_fixed(const ChGroup* g, int z);
 // Sets up the Cahn-Hilliard-Cook deviates of the group's next step for its
 // first gact slots (slot z: key (seed, sim0 + z)), into rho (2 nx ny doubles
 // per slot): drawn in place by the FP64 right-hand side when nx is even,

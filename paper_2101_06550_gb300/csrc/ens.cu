@@ -415,6 +415,8 @@ extern "C" int ens_slot_move(chx_ens* e, int group_id, int from, int to, void* s
   const size_t nb = (size_t)G->n * G->n * sizeof(double);
   cudaStream_t st = (cudaStream_t)stream;
   int rc = CHX_OK;
+  // the captured launches are those of the old slot's kind of operator
+  if (group_slot_fixed(&G->g, from) != group_slot_fixed(&G->g, to)) drop_graph(e);
   for (int b = 0; b < 2 && !rc; ++b)
     rc = cuda_check(cudaMemcpyAsync((char*)G->d_state[b] + to * nb, (char*)G->d_state[b] + from * nb, nb,
                                     cudaMemcpyDeviceToDevice, st),

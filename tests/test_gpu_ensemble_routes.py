@@ -1,0 +1,75 @@
+"""FP64 ensembles whose slots take different solves: fixed point where the operators have circulant
+tables, LU for no implicit part (gamma = 0) and for stiff operators (a' > 5e4)."""
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+N, DT = 64, 1e-3
+SIDE = N * 2 * np.pi / 256
+DX = SIDE / N
+ORDINARY = [0.005, 0.01, 0.02]
+STIFF = 6e4 * DX**4 / (2 / 3 * DT)  # a' = 6e4
+
+
+def _chx():
+    import paper_2101_06550_gb300 as chx
+
+    return chx
+
+
+def _ic(seed):
+    """A few long waves: the implicit part of a step is as large as the field, not a' times larger."""
+    a, b = 2 * np.pi * synth.uniform(seed, 2, 0, 1)
+    x = 2 * np.pi * np.arange(N) / N
+    return torch.from_numpy(0.3 * np.cos(x + a)[None, :] * np.cos(2 * x + b)[:, None] + 0.1).cuda()
+
+
+def _read(ens, gid, slot):
+    out = torch.empty((N, N), dtype=torch.float64, device="cuda")
+    ens.read(gid, slot, out)
+    return out
+
+
+def _lone(seed, gamma, steps):
+    """The simulation as a plan of its own."""
+    chx = _chx()
+    plan = chx.ChPlan(N, N, SIDE, SIDE, gamma, DT, chx.PREC_F64)
+    now = _ic(seed)
+    prev = now.clone()
+    plan.step(now, prev, plan.alloc_work(), steps)
+    torch.cuda.synchronize()
+    return now
+
+
+def _close(a, b):
+    # a step's two solves differ by rounding (1e-11, tests/test_gpu_ch.py) and a few steps carry it on
+    assert torch.max(torch.abs(a - b)) <= 5e-11 * torch.max(torch.abs(b))
+
+
+@pytest.mark.parametrize("gamma", [0.0, STIFF])
+@pytest.mark.parametrize("steps", [2, 3])
+def test_slot_moved_onto_an_active_one_after_capture(gamma, steps):
+    """The captured steps belong to the slots' operators: a slot of the other kind moved onto an
+    active one takes its own operator along, in pairs of steps (replayed) and single ones alike."""
+    ens = _chx().Ensemble(DT, _chx().PREC_F64)
+    gid = ens.group_create(N, SIDE, ORDINARY[1], 3)
+    for s, g in enumerate([ORDINARY[0], ORDINARY[2], gamma]):
+        ens.load(gid, s, _ic(10 + s), None, g)
+    ens.set_active(gid, 2)
+    ens.step(2)
+    ens.move(gid, 2, 1)
+    ens.step(steps)
+    _close(_read(ens, gid, 0), _lone(10, ORDINARY[0], 2 + steps))
+    _close(_read(ens, gid, 1), _lone(12, gamma, steps))
+    # and back: an ordinary slot onto the one that LU serves
+    ens.load(gid, 2, _ic(20), None, ORDINARY[2])
+    ens.step(2)
+    ens.move(gid, 2, 1)
+    ens.step(steps)
+    _close(_read(ens, gid, 0), _lone(10, ORDINARY[0], 4 + 2 * steps))
+    _close(_read(ens, gid, 1), _lone(20, ORDINARY[2], steps))
+    ens.sync_status()
