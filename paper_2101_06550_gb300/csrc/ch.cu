@@ -1071,7 +1071,15 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   // 90, 100; 2048 x 300 53, 79; 2048^2 161, 180).
   g->single = single;
   const bool refine = single && (size_t)nx * ny <= 1u << 20 && nx <= 1400 && ny <= 1400;
-  g->fused = (precision == CHX_PREC_F64 || refine) && adi_shape(nx, ny, G, &g->adi);
+  // Groups of many small fields fill the chip with the LU solves' one thread per segment, and
+  // the fixed-point blocks' barriers and sweeping quarter then cost more than their latency
+  // saves.  us per FP64 step, LU against fixed point: 64^2 x 64 45, 38, x 128 58, 59, x 1024
+  // 280, 400; 33^2 x 128 63, 46, x 512 106, 139; 96^2 x 64 60, 61, x 256 172, 200; 128^2 x 64
+  // 90, 76, x 512 534, 541; from 192^2 on fixed point is level or ahead at any count (192^2 x
+  // 768 1752, 1760; 200^2 x 768 2146, 1985; 384^2 x 192 1738, 1532).  By the capacity, not the
+  // active count: a simulation's arithmetic does not depend on the others.
+  const bool many = G > 128 && nx < 192 && ny < 192;
+  g->fused = ((precision == CHX_PREC_F64 && !many) || refine) && adi_shape(nx, ny, G, &g->adi);
   if (g->fused) {
     g->X.cP = g->adi.xP, g->X.cm = g->adi.xm;
     g->Y.cP = g->adi.yP, g->Y.cm = g->adi.ym;

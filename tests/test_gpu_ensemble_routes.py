@@ -73,3 +73,28 @@ def test_slot_moved_onto_an_active_one_after_capture(gamma, steps):
     _close(_read(ens, gid, 0), _lone(10, ORDINARY[0], 4 + 2 * steps))
     _close(_read(ens, gid, 1), _lone(20, ORDINARY[2], steps))
     ens.sync_status()
+
+
+@pytest.mark.parametrize("n,capacity", [(33, 128), (33, 129), (191, 129), (192, 129)])
+def test_both_sides_of_the_rule_for_many_small_fields(n, capacity):
+    """Fixed point up to 128 slots or from 192 points a side on, LU beyond."""
+    chx = _chx()
+    side = n * DX
+    x = 2 * np.pi * np.arange(n) / n
+    ens = chx.Ensemble(DT, chx.PREC_F64)
+    gid = ens.group_create(n, side, 0.01, capacity)
+    first = torch.from_numpy(0.3 * np.cos(x)[None, :] * np.sin(2 * x)[:, None] + 0.1).cuda()
+    last = first.T.contiguous() - 0.2
+    for s in range(capacity):
+        ens.load(gid, s, first if s == 0 else last)
+    ens.set_active(gid, capacity)
+    ens.step(3)
+    ens.sync_status()
+    plan = chx.ChPlan(n, n, side, side, 0.01, DT, chx.PREC_F64)
+    work = plan.alloc_work()
+    for slot, c in ((0, first), (capacity - 1, last)):
+        now, prev = c.clone(), c.clone()
+        plan.step(now, prev, work, 3)
+        out = torch.empty((n, n), dtype=torch.float64, device="cuda")
+        ens.read(gid, slot, out)
+        _close(out, now)
