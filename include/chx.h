@@ -340,7 +340,9 @@ int cn1d_step(chx_cn1d_plan* plan, double* c, int nsteps, void* stream);
  *    group would take the ensemble past hbm_budget_bytes (0 = no budget).
  *  - Slots [0, active) of each group are stepped (ens_group_set_active); the
  *    caller keeps active simulations packed with ens_slot_move.  A simulation's
- *    arithmetic does not depend on which other slots are active.
+ *    arithmetic does not depend on which other slots are active: where an FP64
+ *    group mixes operators of ch_step's two kinds (gamma = 0 or a' > 5e4 beside
+ *    others), both sets of kernels run, each on its own slots.
  *  - ens_step advances every active slot of every group by nsteps, replaying a
  *    CUDA graph that holds two steps of all groups (one graph branch per
  *    group); the graph is rebuilt after any change of groups or active counts.

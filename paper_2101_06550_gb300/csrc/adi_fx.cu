@@ -313,6 +313,7 @@ struct Walk {
 // the threads of a warp, one segment each, then touch different banks).
 template <int NT>
 __global__ void __launch_bounds__(NT) adi_x_kernel(AdiStep P) {
+  if (P.on && !P.on[blockIdx.y]) return;
   extern __shared__ long long sm[];
   FxShared* sh = (FxShared*)sm;
   long long* e = sm + kHead;
@@ -379,6 +380,7 @@ inline __host__ __device__ int y_pitch(int S, int m) { return m * S + (S <= 8 ? 
 // sweeps made it slower, 84 against 81 us.)
 template <int NT>
 __global__ void __launch_bounds__(NT) adi_y_kernel(AdiStep P, double* cn, double* cp, int keep_roles) {
+  if (P.on && !P.on[blockIdx.y]) return;
   extern __shared__ long long sm[];
   FxShared* sh = (FxShared*)sm;
   long long* e = sm + kHead;

@@ -94,6 +94,9 @@ __device__ __forceinline__ int wrap_near(int i, int n) {
 }
 
 // ---------------------------------------------------------------------------
+// (The LU step's kernels take `fx`: flags of the group's slots that step in fixed point and are
+// left alone here; nullptr when there are none.)
+//
 // The FP64 right-hand side, in two passes over 32 (i) x 32 (j) tiles of
 // simulation blockIdx.z (gls[z] = gamma / dx^2):
 //   pass 1 (ch_rhs_m_kernel): Cbar = 2 C^n - C^{n-1} with a 1-point halo, then
@@ -115,7 +118,9 @@ template <typename TC>
 __global__ void __launch_bounds__(kT* kRBY, kRMMinBlocks) ch_rhs_m_kernel(const double* __restrict__ cn,
                                                             const double* __restrict__ cp, double* __restrict__ m,
                                                             double* __restrict__ cbar, int nx, int ny, TC rho,
-                                                            TC kap, const TC* __restrict__ gls) {
+                                                            TC kap, const TC* __restrict__ gls,
+                                                            const int* __restrict__ fx) {
+  if (fx && fx[blockIdx.z]) return;
   __shared__ TC s_cb[kT + 2][kT + 3];
   const int z = blockIdx.z;
   const TC gl = gls[z];
@@ -182,9 +187,10 @@ __global__ void __launch_bounds__(kT* kRBY, kRLapMinBlocks) ch_rhs_r_kernel(cons
                                                             const double* __restrict__ cn,
                                                             const double* __restrict__ cbar, TO* __restrict__ rT,
                                                             int nx, int ny, int G, TC rho, TC kap, TC kd,
-                                                            double* dev = nullptr, double nkx = 0, double nky = 0,
+                                                            const int* __restrict__ fx, double* dev = nullptr, double nkx = 0, double nky = 0,
                                                             uint64_t seed = 0, uint64_t sim0 = 0, uint64_t step = 0,
                                                             const uint64_t* __restrict__ d_step = nullptr) {
+  if (fx && fx[blockIdx.z]) return;
   __shared__ TC s_m[kT + 2][kT + 3];
   __shared__ TC s_d[kT][kT + 1];
   __shared__ TC s_nz[NOISE == kNoiseRead ? kT : 1][kT + 1];
@@ -275,11 +281,12 @@ __global__ void __launch_bounds__(kT* kRBY, kRLapMinBlocks) ch_rhs_r_kernel(cons
 template <typename TIn, typename TC, int U = (sizeof(TC) == 8 ? 8 : 32)>
 __global__ void __launch_bounds__(kSolveThreads) spike_local_kernel(const TIn* f, TC* y, int ld, int nsys,
                                                                     DirView<TC> D, TC* __restrict__ yb, size_t fz,
-                                                                    size_t ybz) {
+                                                                    size_t ybz, const int* __restrict__ fx) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nsys) return;
   const int s = blockIdx.y, m = D.m;
   const int slot = blockIdx.z + j / D.spp;
+  if (fx && fx[slot]) return;
   const TC a = D.a[slot];
   const TC* lu = D.lu + (size_t)slot * 4 * m;
   f += blockIdx.z * fz;
@@ -359,11 +366,13 @@ __global__ void __launch_bounds__(kSolveThreads) spike_local_kernel(const TIn* f
 template <typename TC, int U = 8>
 __global__ void __launch_bounds__(kSolveThreads) spike_local_even_kernel(const TC* f, TC* y, int ld, int nsys,
                                                                          DirView<TC> D, TC* __restrict__ yb,
-                                                                         size_t fz, size_t ybz) {
+                                                                         size_t fz, size_t ybz,
+                                                                         const int* __restrict__ fx) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nsys) return;
   const int s = blockIdx.y, m = D.m;
   const int slot = blockIdx.z + j / D.spp;
+  if (fx && fx[slot]) return;
   const TC a = D.a[slot];
   const TC* lu = D.lu + (size_t)slot * 4 * m;
   f += blockIdx.z * fz;
@@ -450,12 +459,13 @@ __global__ void __launch_bounds__(kSolveThreads) spike_local_even_kernel(const T
 template <typename TC, int R>
 __global__ void __launch_bounds__(kSolveThreads) spike_reducedR_kernel(const TC* __restrict__ yb, DirView<TC> D,
                                                                        TC* __restrict__ tau, int nsys, size_t ybz,
-                                                                       TC scale) {
+                                                                       TC scale, const int* __restrict__ fx) {
   static_assert(R == 1 || R == 2 || R == 4, "rows per thread");
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nsys) return;
   const int P = D.P, k = 4 * P;
   const int slot = blockIdx.z + j / D.spp;
+  if (fx && fx[slot]) return;
   yb += blockIdx.z * ybz;
   tau += blockIdx.z * ybz;
   const int sq = blockIdx.y / (4 / R), q0 = 4 * sq + (blockIdx.y % (4 / R)) * R;  // first output row
@@ -508,7 +518,9 @@ __device__ __forceinline__ TC spike_apply(TC y, const TC* __restrict__ vw, const
 // y[i*(G*ny) + z*ny + j]) -> w[z*nx*ny + j*nx + i].
 template <typename TC, typename TO>
 __global__ void __launch_bounds__(kT* kBY) ch_xfinish_kernel(const TC* __restrict__ y1, const TC* __restrict__ t1,
-                                                             DirView<TC> D, TO* __restrict__ w, int nx, int ny, int G) {
+                                                             DirView<TC> D, TO* __restrict__ w, int nx, int ny, int G,
+                                                             const int* __restrict__ fx) {
+  if (fx && fx[blockIdx.z]) return;
   __shared__ TO s_t[kT][kT + 1];
   const int z = blockIdx.z, m = D.m, P = D.P;
   const TC* vw = D.vw + (size_t)z * 4 * m;
@@ -543,10 +555,10 @@ template <typename TC>
 __global__ void __launch_bounds__(kSolveThreads) ch_update_kernel(const TC* __restrict__ y1, const TC* __restrict__ t1,
                                                                   DirView<TC> D, const double* __restrict__ cbar,
                                                                   double* cn, double* cp, int nx, int ny, double k2,
-                                                                  int keep_roles) {
+                                                                  int keep_roles, const int* __restrict__ fx) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y, z = blockIdx.z, m = D.m, P = D.P;
-  if (i >= nx) return;
+  if (i >= nx || (fx && fx[z])) return;
   const int s = j / m, r = j - s * m;
   const size_t p = (size_t)z * nx * ny + (size_t)j * nx + i;
   t1 += (size_t)z * 4 * P * nx;
@@ -1020,6 +1032,8 @@ static int group_move_params_gl(ChGroup* g, int from, int to) {
   int rc = cuda_check(cudaMemcpy(g->d_gl + to, g->d_gl + from, 8, cudaMemcpyDeviceToDevice), "ch: replicate");
   if (!rc && g->d_fxgl)
     rc = cuda_check(cudaMemcpy(g->d_fxgl + to, g->d_fxgl + from, sizeof(FxGl), cudaMemcpyDeviceToDevice), "ch: replicate");
+  if (!rc && g->d_fixed)
+    rc = cuda_check(cudaMemcpy(g->d_fixed + to, g->d_fixed + from, sizeof(int), cudaMemcpyDeviceToDevice), "ch: replicate");
   if (!rc) rc = cuda_check(cudaMemcpy(g->d_glff + to, g->d_glff + from, 8, cudaMemcpyDeviceToDevice), "ch: replicate");
   return rc;
 }
@@ -1083,7 +1097,8 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   if (g->fused) {
     g->X.cP = g->adi.xP, g->X.cm = g->adi.xm;
     g->Y.cP = g->adi.yP, g->Y.cm = g->adi.ym;
-    if ((rc = dev_alloc(&g->X.d_circ, G)) || (rc = dev_alloc(&g->Y.d_circ, G)) || (rc = dev_alloc(&g->d_fxgl, G))) {
+    if ((rc = dev_alloc(&g->X.d_circ, G)) || (rc = dev_alloc(&g->Y.d_circ, G)) || (rc = dev_alloc(&g->d_fxgl, G)) ||
+        (rc = dev_alloc(&g->d_fixed, G))) {
       group_free(g);
       return rc;
     }
@@ -1104,7 +1119,7 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
       const size_t m4 = 4 * (size_t)D.m, kk = (size_t)16 * D.P * D.P;
       return (size_t)G * ((D.d_circ ? sizeof(FxDir) : 0) + 8 + 4 + 8 + m4 * (8 + 8 + 4 + 4 + 4 + 4 + 4) + kk * (8 + 4 + 4 + 4 + 4));
     };
-    g->factor_bytes = dir_bytes(g->X) + dir_bytes(g->Y) + (size_t)G * (sizeof(double) + sizeof(float2) + (g->fused ? sizeof(FxGl) : 0));
+    g->factor_bytes = dir_bytes(g->X) + dir_bytes(g->Y) + (size_t)G * (sizeof(double) + sizeof(float2) + (g->fused ? sizeof(FxGl) + sizeof(int) : 0));
   }
   for (int z = 1; z < G && !rc; ++z) rc = group_move_params_gl(g, 0, z);
   if (rc) {
@@ -1157,7 +1172,9 @@ int group_set_gamma(ChGroup* g, int z, double gamma) {
   if (z == 0) g->gamma = gamma;
   if (g->d_fxgl) {
     const FxGl fxgl = fx_gl_host(gl, gamma / (g->dy * g->dy));
-    if ((rc = cuda_check(cudaMemcpy(g->d_fxgl + z, &fxgl, sizeof(fxgl), cudaMemcpyHostToDevice), "ch: gamma upload")))
+    const int fixed = group_slot_fixed(g, z);
+    if ((rc = cuda_check(cudaMemcpy(g->d_fxgl + z, &fxgl, sizeof(fxgl), cudaMemcpyHostToDevice), "ch: gamma upload")) ||
+        (rc = cuda_check(cudaMemcpy(g->d_fixed + z, &fixed, sizeof(fixed), cudaMemcpyHostToDevice), "ch: gamma upload")))
       return rc;
   }
   return cuda_check(cudaMemcpy(g->d_glff + z, &glff, sizeof(float2), cudaMemcpyHostToDevice), "ch: gamma upload");
@@ -1169,6 +1186,9 @@ int group_move_params(ChGroup* g, int from, int to, cudaStream_t st) {
   if ((rc = dir_move(&g->X, from, to, st)) || (rc = dir_move(&g->Y, from, to, st))) return rc;
   if (g->d_fxgl && (rc = cuda_check(cudaMemcpyAsync(g->d_fxgl + to, g->d_fxgl + from, sizeof(FxGl),
                                                     cudaMemcpyDeviceToDevice, st), "ch: move")))
+    return rc;
+  if (g->d_fixed && (rc = cuda_check(cudaMemcpyAsync(g->d_fixed + to, g->d_fixed + from, sizeof(int),
+                                                     cudaMemcpyDeviceToDevice, st), "ch: move")))
     return rc;
   if ((rc = cuda_check(cudaMemcpyAsync(g->d_gl + to, g->d_gl + from, 8, cudaMemcpyDeviceToDevice, st), "ch: move")))
     return rc;
@@ -1183,7 +1203,9 @@ void group_free(ChGroup* g) {
   cudaFree(g->d_gl);
   cudaFree(g->d_glff);
   cudaFree(g->d_fxgl);
+  cudaFree(g->d_fixed);
   g->d_fxgl = nullptr;
+  g->d_fixed = nullptr;
   g->d_gl = nullptr;
   g->d_glff = nullptr;
 }
@@ -1192,13 +1214,13 @@ void group_free(ChGroup* g) {
 // per system, not load latency, limits these sweeps; a shared-memory staged
 // variant measured 82 us against 51 us at 2048^2).
 static void launch_local(const double* f, double* y, int ld, int nsys, const DirView<double>& D, double* yb, size_t fz,
-                         size_t ybz, int Z, cudaStream_t st) {
+                         size_t ybz, int Z, const int* fx, cudaStream_t st) {
   const unsigned blk = balanced_block((size_t)nsys * D.P * Z);
   const dim3 grid(ceil_div(nsys, blk), D.P, Z);
   if (D.m % 16 == 0)
-    spike_local_even_kernel<double><<<grid, blk, 0, st>>>(f, y, ld, nsys, D, yb, fz, ybz);
+    spike_local_even_kernel<double><<<grid, blk, 0, st>>>(f, y, ld, nsys, D, yb, fz, ybz, fx);
   else
-    spike_local_kernel<double, double><<<grid, blk, 0, st>>>(f, y, ld, nsys, D, yb, fz, ybz);
+    spike_local_kernel<double, double><<<grid, blk, 0, st>>>(f, y, ld, nsys, D, yb, fz, ybz, fx);
 }
 
 // FP64 reduced solves: kReducedRows rows per thread, in single-warp blocks when
@@ -1207,23 +1229,24 @@ static void launch_local(const double* f, double* y, int ld, int nsys, const Dir
 // threads hide more load latency (measured 10.4 us against 14 us at 2048^2).
 template <typename TC>
 static void launch_reduced(const TC* yb, const DirView<TC>& D, TC* tau, int nsys, size_t ybz, int Z, TC scale,
-                           cudaStream_t st) {
+                           const int* fx, cudaStream_t st) {
   const int R = kReducedRows;
   const unsigned blk = balanced_block((size_t)nsys * D.P * (4 / R) * Z);
   spike_reducedR_kernel<TC, kReducedRows><<<dim3(ceil_div(nsys, blk), D.P * (4 / R), Z), blk, 0, st>>>(
-      yb, D, tau, nsys, ybz, scale);
+      yb, D, tau, nsys, ybz, scale, fx);
 }
 
 // The step in fixed-point arithmetic (fx.cuh): three launches.  FP32+refine groups have
 // the same space in the pairs of FP32 arrays of r and w.
-static void step_fused(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
-                    Prof* prof) {
+// on: flags of the slots to step (nullptr: all).
+static void step_fused(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, const int* on,
+                       cudaStream_t st, Prof* prof) {
   const AdiShape& s = g->adi;
   double* f = wptr<double>(work, g->off_f);
   int* wtop = wptr<int>(work, g->off_cb);  // G, then the units
-  const FxRhs R{g->nx, g->ny, G, g->d_fxgl, g->rho, g->k1 / g->k2, f, wtop, g->noise, g->noise_w, g->nkx / g->k2,
+  const FxRhs R{g->nx, g->ny, G, on, g->d_fxgl, g->rho, g->k1 / g->k2, f, wtop, g->noise, g->noise_w, g->nkx / g->k2,
                 g->nky / g->k2, g->noise_seed, g->noise_sim0, g->noise_step, g->noise_dstep};
-  const AdiStep P{g->nx, g->ny, G, s.xr, s.xP, s.xm, s.ys, s.yP, s.ym, g->X.d_circ, g->Y.d_circ, f,
+  const AdiStep P{g->nx, g->ny, G, on, s.xr, s.xP, s.xm, s.ys, s.yP, s.ym, g->X.d_circ, g->Y.d_circ, f,
                  wptr<long long>(work, g->off_w), wtop + G, wtop, g->k2};
   { PROF(kRhs); launch_fx_rhs(R, cur, prev, st); }
   { PROF(kXSolve); launch_adi_x(P, s, st); }
@@ -1232,15 +1255,15 @@ static void step_fused(ChGroup* g, int G, double* cur, double* prev, void* work,
 
 bool group_slot_fixed(const ChGroup* g, int z) { return g->fused && g->X.circ_ok[z] && g->Y.circ_ok[z]; }
 
-// Whether the first G slots' operators all have circulant tables.
-static bool fused_serves(const ChGroup* g, int G) {
-  for (int z = 0; z < G; ++z)
-    if (!group_slot_fixed(g, z)) return false;
-  return true;
+// How many of the first G slots step in fixed point.
+static int fixed_slots(const ChGroup* g, int G) {
+  int n = 0;
+  for (int z = 0; z < G; ++z) n += group_slot_fixed(g, z);
+  return n;
 }
 
-static void step_f64(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
-                     Prof* prof, int* status) {
+static void step_f64(ChGroup* g, int G, double* cur, double* prev, void* work, int keep_roles, const int* fx,
+                     cudaStream_t st, Prof* prof) {
   const int nx = g->nx, ny = g->ny;
   const size_t N = (size_t)nx * ny;
   double* f = wptr<double>(work, g->off_f);
@@ -1254,28 +1277,28 @@ static void step_f64(ChGroup* g, int G, double* cur, double* prev, void* work, i
   const size_t kyz = 4 * (size_t)Y.P * nx;
   double* mf = wptr<double>(work, g->off_m);
   { PROF(kRhs); ch_rhs_m_kernel<double><<<tgrid, rblock, 0, st>>>(cur, prev, mf, cbar, nx, ny, g->rho, g->kap,
-                                                                  g->d_gl); }
+                                                                  g->d_gl, fx); }
   {
     PROF(kRhsLap);
     const double kd = g->k1 / g->k2;
     if (g->noise_w)
       ch_rhs_r_kernel<double, double, kNoiseDraw><<<tgrid, rblock, 0, st>>>(
-          mf, cur, cbar, f, nx, ny, G, g->rho, g->kap, kd, g->noise_w, g->nkx / g->k2, g->nky / g->k2,
+          mf, cur, cbar, f, nx, ny, G, g->rho, g->kap, kd, fx, g->noise_w, g->nkx / g->k2, g->nky / g->k2,
           g->noise_seed, g->noise_sim0, g->noise_step, g->noise_dstep);
     else if (g->noise)
       ch_rhs_r_kernel<double, double, kNoiseRead><<<tgrid, rblock, 0, st>>>(
-          mf, cur, cbar, f, nx, ny, G, g->rho, g->kap, kd, const_cast<double*>(g->noise), g->nkx / g->k2,
+          mf, cur, cbar, f, nx, ny, G, g->rho, g->kap, kd, fx, const_cast<double*>(g->noise), g->nkx / g->k2,
           g->nky / g->k2);
     else
-      ch_rhs_r_kernel<double, double><<<tgrid, rblock, 0, st>>>(mf, cur, cbar, f, nx, ny, G, g->rho, g->kap, kd);
+      ch_rhs_r_kernel<double, double><<<tgrid, rblock, 0, st>>>(mf, cur, cbar, f, nx, ny, G, g->rho, g->kap, kd, fx);
   }
-  { PROF(kLocX); launch_local(f, f, nsx, nsx, X, ybx, 0, 0, 1, st); }
-  { PROF(kRedX); launch_reduced<double>(ybx, X, tx, nsx, 0, 1, 1.0, st); }
-  { PROF(kFinX); ch_xfinish_kernel<double, double><<<tgrid, tblock, 0, st>>>(f, tx, X, w, nx, ny, G); }
-  { PROF(kLocY); launch_local(w, w, nx, nx, Y, yby, N, kyz, G, st); }
-  { PROF(kRedY); launch_reduced<double>(yby, Y, ty, nx, kyz, G, g->k2, st); }
+  { PROF(kLocX); launch_local(f, f, nsx, nsx, X, ybx, 0, 0, 1, fx, st); }
+  { PROF(kRedX); launch_reduced<double>(ybx, X, tx, nsx, 0, 1, 1.0, fx, st); }
+  { PROF(kFinX); ch_xfinish_kernel<double, double><<<tgrid, tblock, 0, st>>>(f, tx, X, w, nx, ny, G, fx); }
+  { PROF(kLocY); launch_local(w, w, nx, nx, Y, yby, N, kyz, G, fx, st); }
+  { PROF(kRedY); launch_reduced<double>(yby, Y, ty, nx, kyz, G, g->k2, fx, st); }
   { PROF(kUpd); ch_update_kernel<double><<<dim3(ceil_div(nx, kSolveThreads), ny, G), kSolveThreads, 0, st>>>(
-        w, ty, Y, cbar, cur, prev, nx, ny, g->k2, keep_roles); }
+        w, ty, Y, cbar, cur, prev, nx, ny, g->k2, keep_roles, fx); }
 }
 
 // FP32 + one refinement pass (Sec. 8's float types): the double-float
@@ -1288,7 +1311,7 @@ static void step_f32r(ChGroup* g, int G, double* cur, double* prev, void* work, 
 
 int group_cook_deviates(ChGroup* g, int gact, double* rho, uint64_t seed, uint64_t sim0, uint64_t step,
                         const uint64_t* d_step, cudaStream_t st) {
-  if ((g->precision == CHX_PREC_F64 || fused_serves(g, gact)) && g->nx % 2 == 0) {
+  if ((g->precision == CHX_PREC_F64 || fixed_slots(g, gact) == gact) && g->nx % 2 == 0) {
     g->noise = nullptr;
     g->noise_w = rho;
     g->noise_seed = seed;
@@ -1310,8 +1333,15 @@ void group_cook_clear(ChGroup* g) {
 
 void group_step(ChGroup* g, int gact, double* cur, double* prev, void* work, int keep_roles, cudaStream_t st,
                 Prof* prof, int* status) {
-  if (fused_serves(g, gact)) step_fused(g, gact, cur, prev, work, keep_roles, st, prof);
-  else if (g->precision == CHX_PREC_F64) step_f64(g, gact, cur, prev, work, keep_roles, st, prof, status);
+  // Slot by slot, so that a simulation takes the same solve whatever its neighbours' operators:
+  // with both kinds among the active slots both sets of launches run, each on its own slots.
+  // They take the work buffer in turn, so such a group pays for both (us per step, all ordinary /
+  // half and half / one LU slot / all LU: 128^2 x 64 76, 125, 120, 90; 512^2 x 8 114, 182, 179, 157).
+  const int fixed = fixed_slots(g, gact);
+  const int* both = fixed && fixed < gact ? g->d_fixed : nullptr;
+  if (fixed) step_fused(g, gact, cur, prev, work, keep_roles, both, st, prof);
+  if (fixed == gact) return;
+  if (g->precision == CHX_PREC_F64) step_f64(g, gact, cur, prev, work, keep_roles, both, st, prof);
   else step_f32r(g, gact, cur, prev, work, keep_roles, st, prof);
 }
 

@@ -176,6 +176,7 @@ struct AdiShape {
 };
 struct AdiStep {
   int nx, ny, G;
+  const int* on;         // per slot, whether to step it (nullptr: all)
   int xr, xP, xm, ys, yP, ym;
   const FxDir *X, *Y;    // per slot
   const double* f;       // right-hand side over k2, row major
@@ -192,6 +193,7 @@ void launch_adi_y(const AdiStep& P, const AdiShape& s, double* cur, double* prev
 // The fixed-point right-hand side (rhs_fx.cu): r / k2, row major, into f.
 struct FxRhs {
   int nx, ny, G;
+  const int* on;         // as AdiStep's
   const FxGl* gl;        // per slot
   double rho, kd;        // dx^2 / dy^2, dx^2 / dt
   double* f;
@@ -254,12 +256,13 @@ struct ChGroup {
   struct ObsState* obs = nullptr;  // observables scratch, made on first use (obs.cu)
   float2* d_glff = nullptr;
   FxGl* d_fxgl = nullptr;                    // slots, with fused
+  int* d_fixed = nullptr;                    // slots, with fused: group_slot_fixed
   SpikeDir X, Y;
   // work layout (byte offsets), for G fields
   size_t off_f = 0, off_flo = 0, off_w = 0, off_wlo = 0, off_y1 = 0, off_y2 = 0, off_x0 = 0, off_cb = 0, off_m = 0;
   size_t off_ybx = 0, off_tx = 0, off_ybx2 = 0, off_tx2 = 0, off_yby = 0, off_ty = 0, off_yby2 = 0, off_ty2 = 0;
   bool single = false;  // a plan's group: its gamma never changes
-  bool fused = false;  // the fused solves' blocks fit (adi); a step takes them when every slot has tables
+  bool fused = false;  // the fused solves' blocks fit (adi); the slots with tables take them
   AdiShape adi{};
   size_t work_bytes = 0;
   size_t factor_bytes = 0;  // device bytes of the per-slot factors and parameters (group_init)

@@ -36,6 +36,7 @@ __device__ __forceinline__ int wrap(int i, int n) {
 template <bool kIso, int NOISE>
 __global__ void __launch_bounds__(kNT, kBlocks) fx_rhs_kernel(FxRhs P, const double* __restrict__ cn,
                                                         const double* __restrict__ cp) {
+  if (P.on && !P.on[blockIdx.z]) return;
   constexpr int kW = kT + 4, kR = kT + 2;
   __shared__ long long s_b[kW][kW + 1];  // Cbar
   __shared__ long long s_m[kR][kR + 1];  // C^n, then M

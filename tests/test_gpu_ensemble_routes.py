@@ -98,3 +98,33 @@ def test_both_sides_of_the_rule_for_many_small_fields(n, capacity):
         out = torch.empty((n, n), dtype=torch.float64, device="cuda")
         ens.read(gid, slot, out)
         _close(out, now)
+
+
+@pytest.mark.parametrize("sigma", [0.0, 1e-8])
+@pytest.mark.parametrize("n", [64, 33])  # even: deviates drawn in the step; odd: before it
+def test_neighbours_of_the_other_solve_change_no_bit(n, sigma):
+    """A simulation alone and beside slots of either kind, in pairs of steps and single ones."""
+    chx = _chx()
+    x = 2 * np.pi * np.arange(n) / n
+    c0 = torch.from_numpy(0.3 * np.cos(x)[None, :] * np.sin(2 * x)[:, None] + 0.1).cuda()
+
+    def run(gammas, slot):
+        ens = chx.Ensemble(DT, chx.PREC_F64)
+        gid = ens.group_create(n, n * DX, 0.01, 5)
+        for s, g in enumerate(gammas):
+            ens.load(gid, s, c0, None, g)
+        ens.set_active(gid, len(gammas))
+        if sigma:
+            ens.set_cook(gid, sigma, 7)
+        ens.step(5)
+        ens.sync_status()
+        out = torch.empty((n, n), dtype=torch.float64, device="cuda")
+        ens.read(gid, slot, out)
+        return out
+
+    # the same slot each time: the forcing goes by the slot
+    mixed = [0.0, 0.013, STIFF, 0.02, 0.0]
+    for slot in range(4):
+        alone = run([0.01] * slot + mixed[slot:slot + 1], slot)
+        assert torch.equal(run(mixed, slot), alone), slot
+    assert torch.equal(run([STIFF, 0.013], 1), run([0.01, 0.013], 1))
