@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(128) ch1d_fx_kernel(double* c, int n, int batc
         ccur = cn;
         return g;
       },
-      [](int) { return 0.0; }, [&](int r, long long y, double) { pc[(size_t)r * B] = fx_to_double(y, S) * sc; });
+      [&](int r, long long y) { pc[(size_t)r * B] = fx_to_double(y, S) * sc; });
 }
 
 }  // namespace
@@ -239,7 +239,7 @@ extern "C" int ch1d_plan_create(chx_ch1d_plan** plan, int n, int batch, double l
   p->alpha = dt / (dx * dx);
   CircFx fx;
   std::vector<int2> h;
-  if (circ_fx_host(n, sigma, 1.0, &fx, &h)) {  // the other forms' tables are not needed then
+  if (circ_fx_host(n, sigma, &fx, &h)) {  // the other forms' tables are not needed then
     const FxGl al = fx_gl_host(p->alpha, 0.0);  // alpha / 2^qa, below 1/2
     p->fx_alpha = al.gx;
     p->fx_qa = al.q;

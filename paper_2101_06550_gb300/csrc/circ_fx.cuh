@@ -1,5 +1,8 @@
-// The circulant sweeps of circulant.cuh in fixed point (fx.cuh) for the 1D time steps'
-// operator 1 + a delta^4: the same two passes with the same closure, a thread per system, in a unit of the system's own.
+// The circulant sweeps of circulant.cuh in fixed point (fx.cuh) for the 1D Cahn-Hilliard
+// step's operator 1 + a delta^4: the same two passes, a thread per system, in a unit of the
+// system's own, so that rounding is relative to a system's largest value.  (Crank-Nicolson
+// hyperdiffusion, a linear solve on data of any range, keeps FP64: over a background of
+// 1e-14 of a peak these sweeps leave it one to three digits, FP64 ten or more.)
 //
 // With |f| <= 2^(59 - hb) in the unit of the forward sweep, 2^hb at least the 1-norm of
 // L^{-1}, no g reaches 2^60; the back sweep's unit is 2^hb times coarser for the same reason
@@ -21,19 +24,19 @@ struct CircFx {
   double scale;
 };
 
-// Tables of 1 + a delta^4 over n rows, the solution to be multiplied by `scale`; false when
-// the fixed-point range does not serve.  h[r] = h_{r-1} 2^-hb.
-bool circ_fx_host(int n, double a, double scale, CircFx* out, std::vector<int2>* h);
+// Tables of 1 + a delta^4 over n rows; false when the fixed-point range does not serve.
+// h[r] = h_{r-1} 2^-hb.
+bool circ_fx_host(int n, double a, CircFx* out, std::vector<int2>* h);
 // Uploads both into one allocation *dst: the CircFx, then h.
 int circ_fx_upload(const CircFx& c, const std::vector<int2>& h, CircFx** dst, const char* what);
 
 #ifdef __CUDACC__
 // load(r) reads what row r needs (r rising, a block ahead), form(that, v1, v2) gives g_r =
-// f_r + k1 g_{r-1} + k2 g_{r-2} from the halves of the two before, out(r, y, a) takes the
-// unscaled solution, a = aux(r) being fetched along with g_r; g is kept at pg + r * B.
-template <typename Load, typename Form, typename Aux, typename Out>
+// f_r + k1 g_{r-1} + k2 g_{r-2} from the halves of the two before, out(r, y) takes the
+// unscaled solution; g is kept at pg + r * B.
+template <typename Load, typename Form, typename Out>
 __device__ __forceinline__ void circ_fx_sweeps(int n, const CircFx* __restrict__ tab, long long* pg, size_t B,
-                                               Load load, Form form, Aux aux, Out out) {
+                                               Load load, Form form, Out out) {
   constexpr int U = kCircU;
   const int2* __restrict__ hh = (const int2*)(tab + 1);
   const int R = tab->R, up = 1 << (30 - tab->hb);
@@ -86,38 +89,32 @@ __device__ __forceinline__ void circ_fx_sweeps(int n, const CircFx* __restrict__
                                tab->closeM[3], vm2, qm));
   const FxVal vs2 = fx_halves(fx_mul(k2, vm2));  // of the closure term -l2 h_r s_2
   long long gb[U];
-  double ab[U];
-  auto fetch = [&](int r0, long long (&g)[U], double (&a)[U]) {
+  auto fetch = [&](int r0, long long (&g)[U]) {
 #pragma unroll
     for (int u = U - 1; u >= 0; --u) {
       const int r = r0 + u;
       g[u] = r >= 0 && r < n ? pg[(size_t)r * B] : 0;
-      a[u] = r >= 0 && r < n ? aux(r) : 0.0;
     }
   };
   auto backward = [&](auto closed, auto full, int r0) {
     long long ng[U];
-    double na[U];
-    fetch(r0 - U, ng, na);
+    fetch(r0 - U, ng);
 #pragma unroll
     for (int u = U - 1; u >= 0; --u) {
       const int r = r0 + u;
       if (decltype(full)::value || r < n) {
         long long y = fx_step(gb[u], up, k1, y1, k2, y2);
         if (decltype(closed)::value) y += fx_mul2(__ldg(&hh[r + 2]), vs1, __ldg(&hh[r + 1]), vs2);
-        out(r, y, ab[u]);
+        out(r, y);
         y2 = y1;
         y1 = fx_halves(y);
       }
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      gb[u] = ng[u];
-      ab[u] = na[u];
-    }
+    for (int u = 0; u < U; ++u) gb[u] = ng[u];
   };
   k = nb - 1;
-  fetch(k * U, gb, ab);
+  fetch(k * U, gb);
   if ((k + 1) * U > n) {
     if (rb == nb) backward(yes, no, k * U);
     else backward(no, no, k * U);

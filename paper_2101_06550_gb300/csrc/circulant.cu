@@ -289,7 +289,7 @@ bool fx_dir_host(int n, int P, int m, double a, FxDir* out) {
   return true;
 }
 
-bool circ_fx_host(int n, double a, double scale, CircFx* out, std::vector<int2>* table) {
+bool circ_fx_host(int n, double a, CircFx* out, std::vector<int2>* table) {
   typedef long double ld;
   Biharmonic F;
   if (n < 3 || !factor_biharmonic(a, &F)) return false;
@@ -347,7 +347,7 @@ bool circ_fx_host(int n, double a, double scale, CircFx* out, std::vector<int2>*
   }
   out->hb = hb;
   out->R = R;
-  out->scale = F.scale * scale;
+  out->scale = F.scale;
   table->assign(R + 3, make_int2(0, 0));
   for (int j = 0; j < R + 3 && j < n + 3; ++j) (*table)[j] = q62(ldexpl(H(j), -hb));
   return true;

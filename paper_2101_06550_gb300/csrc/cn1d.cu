@@ -20,7 +20,6 @@
 #include <vector>
 
 #include "chx_internal.cuh"
-#include "circ_fx.cuh"
 #include "circulant.cuh"
 #include "per_system.cuh"
 
@@ -35,7 +34,6 @@ struct chx_cn1d_plan {
   // Constant: the circulant table (scale 2 / kappa), nullptr when sigma is beyond it and the LU factors serve
   double* d_circ;
   int circ_rows;
-  CircFx* d_fx;   // order 4: its fixed-point form (nullptr: the range does not serve)
   double* d_g;    // forward-sweep scratch, n * batch doubles
   // Rewrite: per-system matrix entries (order + 1 diagonals of n * batch) and a
   // PER_SYSTEM solver plan holding the per-system factors
@@ -211,8 +209,11 @@ __global__ void __launch_bounds__(kThreads) cn_tri_kernel(double* c, double* __r
 // Constant mode through the circulant factorisation (circulant.cuh): the scale
 // 2 / kappa rides on the final 2u - c, so a row takes 5 FP64 operations (9 where
 // the closure reaches) for order 4 and 3 (5) for order 2.  1024 x 65536 on a
-// GB300: hyperdiffusion 1207 -> 832 us, diffusion 749 -> 432 us (40 bytes per
-// row are 400 us of HBM there).
+// GB300: hyperdiffusion 1207 -> 843 us (sigma = 7e3), diffusion 749 -> 432 us (40
+// bytes per row are 400 us of HBM there).  The sweeps in fixed point (circ_fx.cuh)
+// take 709 us, but a linear step's data may hold entries that matter next to others
+// 1e14 times larger: they lost those (1024 rows at sigma = 1, a peak over 1e-14: 4e-3
+// of the background against 1e-14).
 template <int W>
 __global__ void __launch_bounds__(W == 2 ? kMaxBlockWarps * 32 : kThreads) cn_circ_kernel(double* c, double* __restrict__ gs, int n, int batch,
                                                            const double* __restrict__ tab, int R) {
@@ -227,31 +228,6 @@ __global__ void __launch_bounds__(W == 2 ? kMaxBlockWarps * 32 : kThreads) cn_ci
       [&](int r, double g) { pg[(size_t)r * B] = g; }, [&](int r) { return pg[(size_t)r * B]; },
       [&](int r) { return pc[(size_t)r * B]; },
       [&](int r, double y, double cr) { pc[(size_t)r * B] = fma(sc, y, -cr); });
-}
-
-// Order 4 in fixed point (circ_fx.cuh), after a pass over the system for its largest value:
-// the FP64 unit is left with the final 2u - c.  On a GB300: 1024 x 65536 at sigma = 5e4 1015 ->
-// 780 us, 512 x 100000 790 -> 579, 64 x 300000 292 -> 176, 254 x 2848 83 -> 58 (and 1000 x 20000,
-// one warp per scheduler, 372 -> 399).
-__global__ void __launch_bounds__(128) cn_fx_kernel(double* c, long long* __restrict__ gs, int n, int batch,
-                                                    const CircFx* __restrict__ tab) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= batch) return;
-  const size_t B = (size_t)batch;
-  double* pc = c + s;
-  const int E = fx_column_exponent(pc, B, n);
-  if (E == 2047) {
-    for (int r = 0; r < n; ++r) pc[(size_t)r * B] = __longlong_as_double(0x7ff8000000000000ll);
-    return;
-  }
-  const int hb = tab->hb, up = 1 << (30 - hb), S = E - 1022 - 59 + 2 * hb;
-  const int2 k1 = tab->k1, k2 = tab->k2;
-  const double sc = tab->scale;
-  circ_fx_sweeps(
-      n, tab, gs + s, B, [&](int r) { return pc[(size_t)r * B]; },
-      [&](double v, FxVal v1, FxVal v2) { return fx_step(fx_from_double(v, E, 59), up, k1, v1, k2, v2); },
-      [&](int r) { return pc[(size_t)r * B]; },
-      [&](int r, long long y, double cr) { pc[(size_t)r * B] = fma(sc, fx_to_double(y, S), -cr); });
 }
 
 // Rewrite mode: every system's matrix entries, diagonal k of row i at
@@ -287,7 +263,6 @@ void cn1d_plan_free(chx_cn1d_plan* p) {
   if (!p) return;
   if (p->d_fac) cudaFree(p->d_fac);
   if (p->d_circ) cudaFree(p->d_circ);
-  if (p->d_fx) cudaFree(p->d_fx);
   if (p->d_g) cudaFree(p->d_g);
   if (p->d_coef) cudaFree(p->d_coef);
   if (p->penta) penta_plan_free(p->penta);
@@ -369,14 +344,6 @@ extern "C" int cn1d_plan_create(chx_cn1d_plan** plan, int order, int n, int batc
     *plan = p;
     return CHX_OK;
   }
-  CircFx fx;
-  std::vector<int2> h;
-  if (order == 4 && circ_fx_host(n, p->sigma, 2.0, &fx, &h)) {  // the other forms' tables are not needed then
-    rc = circ_fx_upload(fx, h, &p->d_fx, "cn1d_plan_create");
-    if (rc) { cn1d_plan_free(p); return rc; }
-    *plan = p;
-    return CHX_OK;
-  }
   std::vector<double> rows(5 * (size_t)n);
   for (int k = 0; k < 5; ++k)
     for (int i = 0; i < n; ++i) rows[(size_t)k * n + i] = v[k];
@@ -432,9 +399,6 @@ extern "C" int cn1d_step(chx_cn1d_plan* p, double* c, int nsteps, void* stream) 
       else
         tri_per_kernel<double, true><<<ceil_div(p->batch, kPerThreads), kPerThreads, 0, st>>>(
             c, p->d_g, p->n, p->batch, tri_plan_factors(p->tri));
-    } else if (p->d_fx) {
-      const unsigned fblk = blk < 128 ? blk : 128;
-      cn_fx_kernel<<<ceil_div(p->batch, fblk), fblk, 0, st>>>(c, (long long*)p->d_g, p->n, p->batch, p->d_fx);
     } else if (p->d_circ && circ_pays(p->n, p->circ_rows, p->batch, p->order == 4 ? 5 : 3, p->order, p->order == 4 ? 10.0 : 6.0)) {
       if (p->order == 4)
         cn_circ_kernel<2><<<cgrid, cblk, 0, st>>>(c, p->d_g, p->n, p->batch, p->d_circ, p->circ_rows);
