@@ -4,6 +4,7 @@
 #include "fx.cuh"
 
 #include <math.h>
+#include <string.h>
 
 namespace chx {
 namespace {
@@ -92,7 +93,7 @@ bool circ_factor_host(int n, double a_, double b_, double c_, double scale, Circ
   h[1].hi = 1;
   for (int r = 1; r <= n + 1; ++r) {
     h[r + 1] = dd_add(dd_mul(h[r], -l1), dd_mul(h[r - 1], -l2));
-    if (fabs(h[r + 1].hi) < 0x1p-200 && fabs(h[r].hi) < 0x1p-200) break;  // the rest stays 0
+    if (fabs(h[r + 1].hi) < 0x1p-900 && fabs(h[r].hi) < 0x1p-900) break;  // the rest stays 0
   }
   int R = n;
   while (R > 0 && fabs(h[R].hi) < 0x1p-60 && fabs(h[R + 1].hi) < 0x1p-60) --R;
@@ -117,15 +118,27 @@ bool circ_factor_host(int n, double a_, double b_, double c_, double scale, Circ
   const ld M[4] = {(ld)q01.hi + q01.lo, -(ld)l2 * ((ld)q00.hi + q00.lo), (ld)prev.hi + prev.lo,
                    -(ld)l2 * ((ld)qm0.hi + qm0.lo)};
   out->R = R;
-  out->tab.assign(kCircH + R + 3, 0.0);
+  const int nb = (n + kCircU - 1) / kCircU;
+  out->tab.assign(kCircH + n + 3 + (nb + 1) / 2, 0.0);
   double* t = out->tab.data();
   t[0] = -l1, t[1] = -l2, t[2] = (double)(kinv * scale), t[3] = -1.0, t[4] = -2.0;
   for (int k = 0; k < 4; ++k) t[5 + k] = (double)A[k];
   t[9] = (double)(A[0] * M[0] + A[1] * M[2]), t[10] = (double)(A[0] * M[1] + A[1] * M[3]);
   t[11] = (double)(A[2] * M[0] + A[3] * M[2]), t[12] = (double)(A[2] * M[1] + A[3] * M[3]);
-  for (int j = 0; j < R + 3 && j < n + 3; ++j) t[kCircH + j] = h[j].hi + h[j].lo;
-  for (int k = 0; k < (int)out->tab.size(); ++k)
+  for (int j = 0; j < n + 3; ++j) t[kCircH + j] = h[j].hi + h[j].lo;
+  for (int k = 0; k < kCircH + n + 3; ++k)
     if (!isfinite(t[k])) return false;
+  std::vector<int> he(nb);
+  for (int k = 0; k < nb; ++k)
+    for (int j = k * kCircU; j < n + 3 && j <= k * kCircU + kCircU + 1; ++j) {
+      const int e = t[kCircH + j] == 0.0 ? 0 : ilogb(t[kCircH + j]) + 1023;
+      he[k] = e > he[k] ? e : he[k];
+    }
+  int R2 = R;  // the first row from which |h| is below 2^-78
+  while (R2 < n && he[R2 / kCircU] >= 1023 - 78) R2 += kCircU;
+  if (R2 > n) R2 = n;
+  memcpy(t + 14, &R2, sizeof(R2));
+  memcpy(t + kCircH + n + 3, he.data(), nb * sizeof(int));
   return true;
 }
 

@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kThreads) cn_tri_kernel(double* c, double* __r
 // Constant mode through the circulant factorisation (circulant.cuh): the scale
 // 2 / kappa rides on the final 2u - c, so a row takes 5 FP64 operations (9 where
 // the closure reaches) for order 4 and 3 (5) for order 2.  1024 x 65536 on a
-// GB300: hyperdiffusion 1207 -> 843 us (sigma = 7e3), diffusion 749 -> 432 us (40
+// GB300: hyperdiffusion 1207 -> 852 us (sigma = 7e3), diffusion 749 -> 440 us (40
 // bytes per row are 400 us of HBM there).  The sweeps in fixed point (circ_fx.cuh)
 // take 709 us, but a linear step's data may hold entries that matter next to others
 // 1e14 times larger: they lost those (1024 rows at sigma = 1, a peak over 1e-14: 4e-3

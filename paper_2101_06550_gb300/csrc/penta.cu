@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kThreads) penta_solve_kernel(const TIn* in, TW
 
 // UNIFORM rows through the circulant factorisation (circulant.cuh), in place.
 // FP64-pipe bound: 5 to 9 operations per row.  1024 x 65536, a = 7e3, on a GB300:
-// 1066 -> 931 us (LU sweeps with bordering, 9 operations, before).
+// 1066 -> 941 us (LU sweeps with bordering, 9 operations, before).
 __global__ void __launch_bounds__(kMaxBlockWarps * 32) penta_circ_kernel(double* x, int n, int batch,
                                                               const double* __restrict__ tab, int R) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;

