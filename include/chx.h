@@ -57,16 +57,30 @@ enum { CHX_COEF_UNIFORM = 0, CHX_COEF_SHARED = 1, CHX_COEF_PER_SYSTEM = 2 };
 
 enum { CHX_PREMAP_NONE = 0, CHX_PREMAP_CUBIC_MINUS_C = 1 };
 
-/* ch_step precision: plain FP64, or FP32 sweeps with one refinement pass per
- * pentadiagonal solve whose residual, like the right-hand side, is formed in
- * double-float arithmetic (FP64 state and update).  FP32+refine keeps a step
- * within 1e-6 of max|c| of the FP64 step up to a' = (2/3) gamma dt / dx^4 of
- * about 2e4 (the 2048^2, gamma 0.005, dt 5e-4 workload).  Above a' = 5e4 the
- * solves take a second refinement pass: at a' = 3e5 a step from a rough random
- * state is then off by about 5e-6 (smooth states stay within 1e-6).
- * Its fused solves keep whole rows and column strips in shared memory: grids
- * whose rows or columns do not fit are rejected at ch_plan_create with
- * CHX_EUNSUPPORTED. */
+/* ch_step precision.
+ *
+ * CHX_PREC_F64: operators with 2.5e-10 < a' <= 5e4 in both directions, a' =
+ * (2/3) gamma dt / dx^4, are stepped in 64-bit fixed point, others (gamma = 0,
+ * stiffer ones, rows or columns that do not fit in shared memory, ensemble
+ * groups of more than 128 slots of fewer than 192 points a side) by FP64 LU
+ * sweeps.  Accuracy: an error of C^{n+1} is at most 1e-11 max|C^{n+1}| +
+ * 4 eps max|r|, r the step's right-hand side; in fixed point the sweeps' part of
+ * it far from large values is 4 eps max|r| too.  That is relative to the field's
+ * largest value: one exponent serves many values, so entries far below it keep
+ * this absolute accuracy and not their own digits, and values below 2^-895 count
+ * as zero in the implicit part.  (The LU sweeps keep every entry's digits.)
+ *
+ * CHX_PREC_F32_REFINE: FP32 sweeps with one refinement pass per pentadiagonal
+ * solve whose residual, like the right-hand side, is formed in double-float
+ * arithmetic (FP64 state and update).  It keeps a step within 1e-6 of max|c| of
+ * the FP64 step up to a' of about 2e4 (the 2048^2, gamma 0.005, dt 5e-4
+ * workload).  Above a' = 5e4 the solves take a second refinement pass: at a' =
+ * 3e5 a step from a rough random state is then off by about 5e-6 (smooth states
+ * stay within 1e-6).  ch_plan_create plans of up to 2^20 points and 1400 a side
+ * whose operators allow it take the FP64 step in fixed point instead, which is
+ * faster there and far more accurate.  The fused solves keep whole rows and
+ * column strips in shared memory: grids whose rows or columns do not fit are
+ * rejected at ch_plan_create with CHX_EUNSUPPORTED. */
 enum { CHX_PREC_F64 = 0, CHX_PREC_F32_REFINE = 1 };
 
 typedef struct chx_penta_plan chx_penta_plan;
@@ -283,12 +297,16 @@ int chx_coarsening_rate(const double* t, const double* F, int count, double* bet
  *   (I + sigma delta^4) C^{n+1} = C^n + alpha delta^2 (C^3 - C)^n,
  *   sigma = gamma dt / dx^4, alpha = dt / dx^2, dx = l / n
  * (the printed f_i lacks C_i^n; eq6:1Dnumerical has it).  The cyclic
- * pentadiagonal operator is factorised once on the host (FP64, Navon bordering
- * + LU without pivoting) by ch1d_plan_create (n >= 8, batch >= 1, l, dt > 0,
- * gamma >= 0; the plan owns about 9 n doubles of device memory).  ch1d_step
- * advances nsteps >= 0 steps in place on the device array c (n * batch
- * doubles, caller-owned, FP64); it needs no scratch.  Errors: CHX_EINVAL,
- * CHX_ESINGULAR (factorisation), CHX_ENOMEM, CHX_ECUDA.
+ * pentadiagonal operator is factorised once on the host by ch1d_plan_create
+ * (n >= 8, batch >= 1, l, dt > 0, gamma >= 0; the plan owns up to 10 n doubles
+ * of device memory).  ch1d_step advances nsteps >= 0 steps in place on the
+ * device array c (n * batch doubles, caller-owned, FP64); it needs no scratch.
+ * It runs in 64-bit fixed point with one exponent per system (in FP64 for
+ * gamma = 0 and operators outside the fixed-point range): an error is at most
+ * 64 eps max|f| (1 + 16 sigma), 64 eps max|f| far from large values, f a
+ * system's right-hand side; entries far below a system's largest keep that
+ * absolute accuracy and not their own digits, and values below 2^-895 count as
+ * zero.  Errors: CHX_EINVAL, CHX_ESINGULAR (factorisation), CHX_ENOMEM, CHX_ECUDA.
  */
 int ch1d_plan_create(chx_ch1d_plan** plan, int n, int batch, double l, double gamma, double dt);
 int ch1d_step(chx_ch1d_plan* plan, double* c, int nsteps, void* stream);
@@ -307,7 +325,8 @@ int ch1d_step(chx_ch1d_plan* plan, double* c, int nsteps, void* stream);
  * In both the explicit row is twice the identity minus the implicit one
  * (B = 2I - A), so a step is C^{n+1} = 2 A^{-1} C^n - C^n: one cyclic
  * pentadiagonal (Navon bordering + LU) or tridiagonal (Thomas + Sherman-
- * Morrison) solve with right-hand side C^n and no explicit half to form.
+ * Morrison) solve with right-hand side C^n and no explicit half to form, in FP64
+ * throughout: entries keep their digits next to others far larger.
  * cn1d_plan_create: order 2 or 4; n >= 6 (order 4) or >= 3 (order 2);
  * batch >= 1; l, dt > 0; kappa >= 0.  Every plan owns n * batch doubles of
  * sweep scratch.  rewrite selects the paper's benchmark variant (Sec. 4.3):
