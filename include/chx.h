@@ -375,7 +375,8 @@ int cn1d_step(chx_cn1d_plan* plan, double* c, int nsteps, void* stream);
  *    y count held, then every y count with the chosen x count (the two are
  *    independent; px_out / py_out receive them).  The simulations' state is
  *    saved and restored, so the call changes no result other than by rounding
- *    order.
+ *    order.  A group whose active slots all step in fixed point (see
+ *    CHX_PREC_F64) keeps its counts, which only the LU sweeps use.
  *  - ens_group_set_cook turns on the Cahn-Hilliard-Cook forcing of ch_cook_run
  *    (Sec. 7.7) for every slot of a group (either precision): each later step
  *    of the group first draws the deviates of slot s with simulation id s, key

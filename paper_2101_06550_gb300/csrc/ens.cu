@@ -569,6 +569,14 @@ extern "C" int ens_autotune(chx_ens* e, int group_id, int trial, int* px_out, in
   EnsGroup* G = get_group(e, group_id);
   if (!G || trial < 1) return fail(CHX_EINVAL, "ens_autotune: bad argument");
   if (G->active < 1) return fail(CHX_EINVAL, "ens_autotune: group %d has no active slots", group_id);
+  // the fixed-point step has segments of its own: no count to choose while it takes every active slot
+  bool fixed = true;
+  for (int z = 0; z < G->active; ++z) fixed = fixed && group_slot_fixed(&G->g, z);
+  if (fixed) {
+    if (px_out) *px_out = G->g.X.P;
+    if (py_out) *py_out = G->g.Y.P;
+    return CHX_OK;
+  }
   cudaStream_t st = (cudaStream_t)stream;
   const int n = G->n;
   const size_t sb = (size_t)G->active * n * n * sizeof(double);

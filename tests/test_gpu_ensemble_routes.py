@@ -128,3 +128,33 @@ def test_neighbours_of_the_other_solve_change_no_bit(n, sigma):
         alone = run([0.01] * slot + mixed[slot:slot + 1], slot)
         assert torch.equal(run(mixed, slot), alone), slot
     assert torch.equal(run([STIFF, 0.013], 1), run([0.01, 0.013], 1))
+
+
+def test_autotune_where_no_step_reads_the_segment_counts():
+    """All active slots in fixed point: nothing to time, nothing to allocate (a budget without room for
+    a copy of the state), counts and memory as they were.  With an LU slot the counts are chosen."""
+    chx = _chx()
+    free = chx.Ensemble(DT, chx.PREC_F64)
+    free.group_create(N, SIDE, ORDINARY[1], 3)
+    used = free.bytes_used
+    ens = chx.Ensemble(DT, chx.PREC_F64, hbm_budget=used)
+    gid = ens.group_create(N, SIDE, ORDINARY[1], 3)
+    for s, g in enumerate([ORDINARY[0], ORDINARY[2], STIFF]):
+        ens.load(gid, s, _ic(10 + s), None, g)
+    ens.set_active(gid, 2)
+    before = ens.info(gid)
+    assert ens.autotune(gid, 1) == (before["px"], before["py"])
+    assert ens.info(gid) == before and ens.bytes_used == used
+    ens.step(3)
+    _close(_read(ens, gid, 1), _lone(11, ORDINARY[2], 3))
+    ens.set_active(gid, 3)
+    with pytest.raises(chx.ChxError) as e:
+        ens.autotune(gid, 1)
+    assert e.value.status == -4  # the copy of the state is over the budget
+    gid = free.group_create(N, SIDE, ORDINARY[1], 1)
+    free.load(gid, 0, _ic(12), None, STIFF)
+    free.set_active(gid, 1)
+    counts = free.autotune(gid, 1)
+    assert all(N % c == 0 for c in counts)
+    free.step(2)
+    _close(_read(free, gid, 0), _lone(12, STIFF, 2))
