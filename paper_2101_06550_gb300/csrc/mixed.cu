@@ -583,7 +583,7 @@ __device__ __forceinline__ float reduced_row(const float* yb, int q, const float
   auto ld = [](const float* a) { return SH ? *a : __ldg(a); };
   const int K = 4 * P;
   const int nb = 2 * band + 1 < P ? 2 * band + 1 : P;
-  int d = nb == P ? 0 : P - band;  // block offset of the first step (mod P)
+  int d = nb == P || band == 0 ? 0 : P - band;  // block offset of the first step, below P
   int sb = (q >> 2) + d;
   if (sb >= P) sb -= P;
   const size_t stepw = 4 * (size_t)K;
