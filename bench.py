@@ -705,10 +705,15 @@ def bench_ensemble(dev, precision, steps, warmup, count=512, long_steps=2000):
             pc = c.clone()
             w = p64.alloc_work(dev)
             p64.step(c, pc, w, long_steps)
-            # one step of each precision from the FP64 state
-            p32 = chx.ChPlan(n, n, n * dx, n * dx, g, dt, chx.PREC_F32_REFINE)
-            e, f = c.clone(), pc.clone()
-            p32.step(e, f, p32.alloc_work(dev), 1)
+            # one step of each precision from the FP64 state (the ensemble's own kernels: single
+            # FP32+refine plans of these sizes take the FP64 ones)
+            one = chx.Ensemble(dt, precision)
+            gid = one.group_create(n, n * dx, g, 1)
+            one.load(gid, 0, c, pc, g)
+            one.set_active(gid, 1)
+            one.step(1)
+            e = torch.empty(n * n, dtype=torch.float64, device=dev)
+            one.read(gid, 0, e)
             p64.step(c, pc, w, 1)
             torch.cuda.synchronize()
             rows.append({"slot": slot, "gamma": g,
@@ -716,7 +721,7 @@ def bench_ensemble(dev, precision, steps, warmup, count=512, long_steps=2000):
                          "trajectory_rel_err_vs_fp64": float((x - pc).abs().max() / pc.abs().max()),
                          "mass_drift_rel_to_sum_abs_c": abs(float(x.sum()) - m) / sa})
             p64.close()
-            p32.close()
+            one.close()
         acc[n] = rows
     res["accuracy_at_long_steps"] = acc
     ens.close()
