@@ -128,10 +128,12 @@ __global__ void __launch_bounds__(kThreads) ch1d_step_kernel(double* c, int n, i
 }
 
 // The same step through the circulant factorisation (circulant.cuh): 10 FP64
-// operations per row, 14 where the closure reaches, against 14 everywhere.  The
-// constants come from the table, not the parameters: an FP64 instruction with a
-// parameter or immediate operand issues at 0.84 of the full rate.  256 x 262144
-// on a GB300: 1699 -> 1608 us.
+// operations per row, 14 where the closure reaches, against 14 everywhere, for the
+// operators that the fixed-point form declines (next to no implicit part, short and
+// very stiff systems).  The constants come from the table, not the parameters: an
+// FP64 instruction with a parameter or immediate operand issues at 0.84 of the full
+// rate.  256 x 262144 on a GB300, before the fixed-point form took that size: 1699 ->
+// 1608 us.
 __global__ void __launch_bounds__(kMaxBlockWarps * 32) ch1d_circ_kernel(double* c, int n, int batch,
                                                              const double* __restrict__ tab, int R) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;

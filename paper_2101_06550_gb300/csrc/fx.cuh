@@ -177,14 +177,6 @@ __device__ __forceinline__ int fx_bits(int v) { return 32 - __clz(v); }
 __device__ __forceinline__ double fx_pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
 #endif  // __CUDACC__
 
-// Shape of the segments of an n-row system: P of m rows, the last one shorter.
-inline int fx_segments(int n, int most) {
-  int P = n / 8 < most ? n / 8 : most;
-  if (P < 1) P = 1;
-  const int m = (n + P - 1) / P;
-  return (n + m - 1) / m;
-}
-
 // Tables of 1 + a delta^4 over n rows in P segments of m; false when a is next to 0 or stiffer than
 // kFxStiff, or the factorisation or the fixed-point range does not serve (the caller keeps
 // the FP64 solves).  At a = 3e5 (4096^2, a rough state) the circulant factors lose the field's

@@ -190,9 +190,10 @@ __global__ void __launch_bounds__(kPerThreads) tri_per_kernel(T* x, T* gs, int n
 
 // The pivot test |al| > tol (|b0| + .. + |bk|), tol = 1e3 eps, with the exact sum
 // only when exponents cannot settle it: the sum of up to five magnitudes is
-// below 2^(em - 1020) for the largest biased exponent em, so tol times it is
-// below 2^(em - 1061), and an |al| of exponent ea >= em - 38 passes.  (The FP64
-// pipe, which bounds the factorisations, does six operations for the sum.)
+// below 5 * 2^(em - 1022) for the largest biased exponent em, so tol = 2^-42.03
+// times it is below 2^(em - 1061.7), and an |al| of exponent ea >= em - 38, at
+// least 2^(em - 1061), passes.  (The FP64 pipe, which bounds the factorisations,
+// does six operations for the sum.)
 template <int N>
 __device__ __forceinline__ bool pivot_ok(double al, const double (&b)[N]) {
   const int ea = (__double2hiint(al) >> 20) & 0x7ff;
