@@ -1081,8 +1081,8 @@ int group_init(ChGroup* g, int nx, int ny, double lx, double ly, double gamma, d
   int rc;
   // The fixed-point step also serves an FP32+refine plan, more accurately, where it is the
   // faster one: up to 2^20 points and sides of 1400 (us per step, FP32+refine against
-  // fixed point: 128^2 68, 22; 512^2 46, 33; 1024^2 69, 64; 777 x 1311 106, 72; but 1280^2
-  // 90, 100; 2048 x 300 53, 79; 2048^2 161, 180).
+  // fixed point: 128^2 68, 22; 512^2 46, 33; 1024^2 69, 64; 777 x 1311 106, 72; level at 1408 x
+  // 700, 69; but 1280^2 90, 93; 2048 x 300 53, 58; 2048 x 512 67, 69; 2048^2 161, 173).
   g->single = single;
   const bool refine = single && (size_t)nx * ny <= 1u << 20 && nx <= 1400 && ny <= 1400;
   // Groups of many small fields fill the chip with the LU solves' one thread per segment, and
