@@ -10,7 +10,7 @@
 // whose roundings of Cbar the factor gamma / dx^2 enlarges.  The result goes back to
 // FP64 for the difference in time and the forcing: four FP64 operations per point (six
 // with dx != dy), conversions counted, where the two-pass form takes fourteen, at 64
-// cycles per warp each.  2048^2 on a GB300: 49 us, bound by the integer ALU (78% busy),
+// cycles per warp each.  2048^2 on a GB300: 49 us, bound by the integer ALU (71% busy),
 // against 73 + 58 us for the two FP64 passes.
 #include <type_traits>
 
