@@ -2,7 +2,7 @@
 // step's operator 1 + a delta^4: the same two passes, a thread per system, in a unit of the
 // system's own, so that rounding is relative to a system's largest value.  (Crank-Nicolson
 // hyperdiffusion, a linear solve on data of any range, keeps FP64: over a background of
-// 1e-14 of a peak these sweeps leave it one to three digits, FP64 ten or more.)
+// 1e-14 of a peak these sweeps leave it two digits at best, FP64 ten or more.)
 //
 // With |f| <= 2^(59 - hb) in the unit of the forward sweep, 2^hb at least the 1-norm of
 // L^{-1}, no g reaches 2^60; the back sweep's unit is 2^hb times coarser for the same reason
